@@ -124,14 +124,16 @@ void free_vis(ppd_ctx *c) {
     for (void *p : {c->rec, c->theta_v, c->y, c->v, c->z, c->w, c->p, c->y_raw, (void *)c->perm,
                     (void *)c->count_cell, (void *)c->ch.start, (void *)c->ch.count, (void *)c->ch.tile,
                     (void *)c->ch.block, (void *)c->ch.tile_first, (void *)c->ch.tile_n, (void *)c->ch.blk_ptr,
-                    (void *)c->ch.u_start, (void *)c->ch.u_count, (void *)c->ch.u_chunk, (void *)c->ch.u_pos, (void *)c->ch.u_order, (void *)c->ch.order, (void *)c->ch.active, (void *)c->partials, (void *)c->scale, (void *)c->resid2,
-                    (void *)c->eps_d, (void *)c->mu_d, c->gpart})
+                    (void *)c->ch.u_start, (void *)c->ch.u_count, (void *)c->ch.u_chunk, (void *)c->ch.u_pos, (void *)c->ch.u_order, (void *)c->ch.order, (void *)c->ch.active, (void *)c->partials, c->scale, (void *)c->resid2,
+                    (void *)c->eps_d, c->mu_d, (void *)c->blk_done, c->gpart})
         dfree(p);
     c->rec = c->theta_v = c->y = c->v = c->z = c->w = c->p = c->y_raw = c->gpart = nullptr;
     c->perm = nullptr;
     c->count_cell = nullptr;
     c->ch = Chunks{};
-    c->partials = c->scale = c->resid2 = c->eps_d = c->mu_d = nullptr;
+    c->partials = c->resid2 = c->eps_d = nullptr;
+    c->scale = c->mu_d = nullptr;
+    c->blk_done = nullptr;
     c->have_vis = c->have_weights = false;
     c->gpart_stale = true;
 }
@@ -211,8 +213,7 @@ int check_err_word(ppd_ctx *c) {
 // variation of x below tol and every block residual within fac eps_j,
 // evaluated in FP64 on the device; *flag = 1 when it holds (synchronises).
 int stop_rule(ppd_ctx *c, double tol, double fac, int *flag) {
-    c->part_out = c->partials;   // bank 0: the data step's residual partials
-    PPD_CHECK(block_norms(c, 1, c->stream));
+    PPD_CHECK(block_norms(c, c->stream));
     PPD_CHECK(reduce_primal_stats(c, c->stream));
     PPD_CHECK(stop_flag(c, tol, fac, c->stream));
     PPD_CUDA(cudaMemcpyAsync(flag, c->stop_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -224,9 +225,8 @@ int stop_rule(ppd_ctx *c, double tol, double fac, int *flag) {
 // prior branch (SARA analysis, clip, synthesis down to level 1) needs only
 // xt and u, so in the FP32 path it runs on a second stream beside the data
 // branch (FFT, degridding with the data step, gridding, inverse FFT); both
-// join before the primal step.  The per-block P_B
-// scales are computed in the prologue of the kernel that uses them, from the
-// previous launch's chunk partials (two banks).
+// join before the primal step.  The per-block P_B scales are computed by
+// the kernel that forms the norms, in the CTA that finishes a block.
 template <typename R> int iteration_body(ppd_ctx *c, cudaStream_t s, bool first) {
     using C = cplx_t<R>;
     C *ga = static_cast<C *>(c->grid_a), *gv = static_cast<C *>(c->grid_v);
@@ -243,8 +243,6 @@ template <typename R> int iteration_body(ppd_ctx *c, cudaStream_t s, bool first)
     PPD_CHECK(sara_level0<R>(c, ll0, s2));
     if (fork) PPD_CUDA(cudaEventRecord(c->ev_join, s2));
 
-    double *bank[2] = {c->partials, c->partials + NPART * c->ch.nu};
-    int cur = 0;
     // with the fused row kernel the forward row pass of xt was done by the
     // previous iteration's last kernel (or by run_iterations before the first)
     if (!fused_rows(c)) PPD_CHECK(fft_forward_rows<R>(c, static_cast<const R *>(c->xt), s));
@@ -254,8 +252,6 @@ template <typename R> int iteration_body(ppd_ctx *c, cudaStream_t s, bool first)
     // the device (blocks without a prox output start from z, then one extra
     // step gives P_B(z)), so the captured iteration is the same every time
     const bool rnd = c->rand_on;
-    c->part_out = bank[0];
-    c->part_in = bank[1];
     PPD_CHECK(degrid<R>(c, (current || (first && !rnd)) ? DG_FIRST : DG_DUAL, ga, nullptr, nullptr, s));
     // warm start at t = 1: zbar^(0) = P_B(z) (an extra step from z), then
     // the n_itr - 1 steps between the degridding and the gridding; the
@@ -263,12 +259,8 @@ template <typename R> int iteration_body(ppd_ctx *c, cudaStream_t s, bool first)
     // t_1 = 1, from the second of them on
     const bool extra = !current && (rnd || first);
     if (extra) {
-        c->part_in = bank[cur];
-        c->part_out = bank[cur ^ 1];
         c->next_step = 0;
-        c->next_test_in = 0;
         PPD_CHECK(subiter<R>(c, s, /*only_first=*/rnd ? 1 : 0));
-        cur ^= 1;
     }
     const bool fista = c->cfg.inner_solver == PPD_INNER_FISTA;
     double t_k = 1.0;
@@ -276,17 +268,10 @@ template <typename R> int iteration_body(ppd_ctx *c, cudaStream_t s, bool first)
         const double t_next = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t_k * t_k));
         const double beta = fista ? (t_k - 1.0) / t_next : 0.0;
         t_k = t_next;
-        c->part_in = bank[cur];
-        c->part_out = bank[cur ^ 1];
         c->next_step = k;
-        c->next_test_in = k >= 2;   // step k - 1 >= 1 left the test partials
         PPD_CHECK(subiter<R>(c, s, 0, beta, fista ? 1 : 0));
-        cur ^= 1;
     }
-    c->part_in = bank[cur];
-    c->part_out = bank[0];
     c->next_step = c->cfg.n_itr;
-    c->next_test_in = c->cfg.n_itr >= 2;
     // the combine pass sums the partial tiles into the column-major grid,
     // which the inverse column pass reads in whole columns
     PPD_CHECK(grid_vis<R>(c, GR_DUAL, nullptr, nullptr, gv, s));
@@ -544,6 +529,7 @@ int reset_state(ppd_ctx *c) {
         PPD_CUDA(cudaMemsetAsync(c->p, 0, 2 * c->M * rb, c->stream));
     }
     PPD_CUDA(cudaMemsetAsync(c->err, 0, sizeof(int), c->stream));
+    if (c->blk_done) PPD_CUDA(cudaMemsetAsync(c->blk_done, 0, c->d * sizeof(int), c->stream));
     if (c->blk_seen) PPD_CUDA(cudaMemsetAsync(c->blk_seen, 0, c->d, c->stream));
     if (c->inner_state) PPD_CUDA(cudaMemsetAsync(c->inner_state, 0, c->d * sizeof(int), c->stream));
     if (c->inner_steps) PPD_CUDA(cudaMemsetAsync(c->inner_steps, 0, c->d * sizeof(int), c->stream));
@@ -994,9 +980,9 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
         (st = dalloc(&c->ch.u_start, nu)) ||
         (st = dalloc(&c->ch.u_count, nu)) || (st = dalloc(&c->ch.u_chunk, nu)) || (st = dalloc(&c->ch.u_pos, nu)) || (st = dalloc(&c->ch.u_order, nu)) || (st = dalloc(&c->ch.order, nch)) ||
         (st = dalloc(&c->ch.active, active.size())) ||
-        (st = dalloc(&c->partials, 2 * NPART * (size_t)nu)) ||
-        (st = dalloc(&c->scale, c->d)) || (st = dalloc(&c->resid2, c->d)) || (st = dalloc(&c->eps_d, c->d)) ||
-        (st = dalloc(&c->mu_d, c->d)) || (st = dalloc_bytes(&c->gpart, (size_t)nch * E * E * cbsz)) ||
+        (st = dalloc(&c->partials, NPART * (size_t)nu)) ||
+        (st = dalloc_bytes(&c->scale, c->d * c->rsz)) || (st = dalloc(&c->blk_done, c->d)) || (st = dalloc(&c->resid2, c->d)) || (st = dalloc(&c->eps_d, c->d)) ||
+        (st = dalloc_bytes(&c->mu_d, c->d * c->rsz)) || (st = dalloc_bytes(&c->gpart, (size_t)nch * E * E * cbsz)) ||
         (st = dalloc(&c->perm, M)) || (st = dalloc_bytes(&c->rec, M * (c->is_f32 ? 16 : 32))) ||
         (st = dalloc_bytes(&c->y, M * cbsz)) || (st = dalloc_bytes(&c->v, M * cbsz)) ||
         (st = dalloc_bytes(&c->z, M * cbsz)) || (st = dalloc_bytes(&c->w, M * cbsz)) ||
@@ -1145,9 +1131,9 @@ int ppd_set_weights(ppd_ctx *c, const double *theta, const double *U, const doub
         if ((st = dalloc_bytes(&c->theta_v, M * c->rsz))) return st;
         if ((st = c->is_f32 ? upload_real<float>(c->theta_v, th) : upload_real<double>(c->theta_v, th))) return st;
     }
-    if ((e = cudaMemcpy(c->eps_d, ep.data(), c->d * 8, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->mu_d, mu.data(), c->d * 8, cudaMemcpyHostToDevice)))
+    if ((e = cudaMemcpy(c->eps_d, ep.data(), c->d * 8, cudaMemcpyHostToDevice)))
         return fail(PPD_ERR_CUDA, std::string("ppd_set_weights: ") + cudaGetErrorString(e));
+    if ((st = c->is_f32 ? upload_real<float>(c->mu_d, mu) : upload_real<double>(c->mu_d, mu))) return st;
     c->have_weights = true;
     drop_graph(c);
     if ((st = reset_state(c))) return st;
@@ -1225,8 +1211,7 @@ int ppd_iterate(ppd_ctx *c, int32_t n_iters, ppd_stats *stats) {
         return st;
     }
     if (stats) {
-        c->part_out = c->partials;   // bank 0 holds the last data step's residual partials
-        PPD_CHECK(block_norms(c, 1, c->stream));
+        PPD_CHECK(block_norms(c, c->stream));
         PPD_CHECK(reduce_primal_stats(c, c->stream));
         double h[3];
         std::vector<double> r2(c->d);

@@ -208,16 +208,15 @@ struct ppd_ctx {
     std::vector<int64_t> block_count_h;
     int32_t *count_cell = nullptr;   // per visibility (sorted order), device
     ppd::Chunks ch;
-    double *partials = nullptr, *scale = nullptr, *resid2 = nullptr, *eps_d = nullptr,
-           *mu_d = nullptr;
-    double *part_in = nullptr, *part_out = nullptr;   // chunk-partial banks for the next launch
+    double *partials = nullptr, *resid2 = nullptr, *eps_d = nullptr;
+    void *scale = nullptr, *mu_d = nullptr;           // per block, reals: P_B scale of the last step, mu
+    int *blk_done = nullptr;                          // per block: finished work units (zero between launches)
     // Algorithm 2 stopping test (cfg.inner_tol > 0): per block the step at
     // which the test held in the current iteration (0 = still running) and
-    // the steps taken in the last iteration; the arguments of the next
-    // sub-iteration / gridding launch: its step number and whether its input
-    // bank holds the test partials of the previous step
+    // the steps taken in the last iteration; the step number of the next
+    // sub-iteration / gridding launch
     int *inner_state = nullptr, *inner_steps = nullptr;
-    int next_step = 0, next_test_in = 0;
+    int next_step = 0;
     int *stop_flag = nullptr;                          // global stopping rule (device, 1 int)
     int *dg_claim = nullptr;                           // degridding work counters (device, 2 ints, zero between launches)
     cudaStream_t stream2 = nullptr;                   // prior (SARA) branch of the iteration
@@ -325,7 +324,7 @@ int degrid(ppd_ctx *c, int mode, const cplx_t<R> *grid, cplx_t<R> *out, const in
            cudaStream_t s);
 template <typename R>
 int subiter(ppd_ctx *c, cudaStream_t s, int only_first = 0, double beta = 0.0, int write_p = 0);
-int block_norms(ppd_ctx *c, int which, cudaStream_t s);
+int block_norms(ppd_ctx *c, cudaStream_t s);
 template <typename R>
 int grid_vis(ppd_ctx *c, int mode, const cplx_t<R> *in, const int64_t *perm_in, cplx_t<R> *grid,
              cudaStream_t s, bool combine = true);

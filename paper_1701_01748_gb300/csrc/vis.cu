@@ -117,9 +117,10 @@ template <typename R> struct VisArgs {
     double beta, inv_i0b;
     const cplx_t<R> *y;
     cplx_t<R> *v, *z, *w, *p;
-    const double *mu, *scale;
-    double *partials;            // this launch's chunk partials
-    const double *part_in;       // previous step's chunk partials (P_B scale)
+    const R *mu;
+    R *scale;                    // per block: the P_B scale of the last step (block_scale)
+    int *blk_done;               // per block: units of the running launch that are done (zero between launches)
+    double *partials;            // norm partials of the work units
     // partials live in block-major slots: work unit u writes slot
     // u_pos[u]; block b's slots are blk_ptr[b] .. blk_ptr[b+1] - 1
     const int32_t *blk_ptr, *u_pos;
@@ -137,39 +138,36 @@ template <typename R> struct VisArgs {
     const int64_t *perm;
     // Algorithm 2 stopping test (inner_tol > 0): this launch's step number
     // (0: the step that forms the start P_B(z); 1 .. n_itr - 1: sub-iterations;
-    // n_itr: the gridding), whether part_in holds the previous step's test
-    // partials, per block the step at which the test held (0: running) and
-    // the steps taken
+    // n_itr: the gridding), per block the step at which the test held (0:
+    // running) and the steps taken
     double inner_tol;
-    int step, test_in, n_itr;
+    int step, n_itr, n_blocks;
     int *inner_state, *inner_steps;
 };
 
-// Deterministic CTA sum of two doubles per thread (fixed shuffle tree, then
-// warps in order).
-template <int NT> __device__ void cta_sum2(double a, double b, double *out2) {
-    __shared__ double red[2][NT / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-        red[0][wid] = a;
-        red[1][wid] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s0 = 0, s1 = 0;
-        for (int i = 0; i < NT / 32; ++i) {
-            s0 += red[0][i];
-            s1 += red[1][i];
-        }
-        out2[0] = s0;
-        out2[1] = s1;
-    }
+// Unevaluated sum h + l of two floats, |l| <= ulp(h) / 2: about 48 bits, the
+// accumulator of the FP32 path's norm sums inside a CTA (sums over CTAs are
+// in FP64).  The SM has two FP64 lanes, so a warp's FP64 add holds the pipe
+// for 16 cycles where an FP32 one takes a quarter of a cycle of the SM's
+// issue: the ~10 FP32 instructions of one add below are still 6 times less.
+struct F2 {
+    float h, l;
+};
+__device__ __forceinline__ F2 f2add(F2 a, F2 b) {   // two-sum of the heads, then the tails
+    const float s = a.h + b.h, t = s - a.h;
+    float e = (a.h - (s - t)) + (b.h - t);
+    e += a.l + b.l;
+    const float h = s + e;
+    return isfinite(h) ? F2{h, e - (h - s)} : F2{s, 0.f};
 }
+__device__ __forceinline__ F2 shfl_xor_(F2 v, int m) {
+    return F2{__shfl_xor_sync(0xffffffffu, v.h, m), __shfl_xor_sync(0xffffffffu, v.l, m)};
+}
+__device__ __forceinline__ double shfl_xor_(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+__device__ __forceinline__ F2 sum_of(F2 a, F2 b) { return f2add(a, b); }
+__device__ __forceinline__ double sum_of(double a, double b) { return a + b; }
+__device__ __forceinline__ double as_double(F2 v) { return (double)v.h + (double)v.l; }
+__device__ __forceinline__ double as_double(double v) { return v; }
 
 // Kahan-compensated FP32 accumulator (FP64 accumulation in the FP64 path).
 template <typename R> struct Acc {
@@ -180,69 +178,100 @@ template <typename R> struct Acc {
         c = (t - s) - y;
         s = t;
     }
-    __device__ double get() const { return (double)s - (double)c; }
+    __device__ auto get() const {   // s - c, unrounded
+        if constexpr (sizeof(R) == 4) {
+            const float h = s - c;
+            return isfinite(h) ? F2{h, (s - h) - c} : F2{s, 0.f};
+        } else {
+            return s - c;
+        }
+    }
 };
+
+// Deterministic CTA sums of NV <= 4 values per thread.  The first shuffle
+// steps also halve the number of values a lane carries (lanes whose bit is
+// set take the upper half), so that NV = 2 costs 5 adds a lane instead of
+// 10; then the warps' sums in a fixed tree.  The sums are valid in thread 0
+// after the call (out[k]); the CTA must pass a barrier before `red` is used
+// again by another call.
+template <int NT, int NV, typename V> __device__ __forceinline__ void cta_sums(const V (&in)[NV], double (&out)[NV]) {
+    constexpr int NW = NT / 32, NP = NV <= 1 ? 1 : NV <= 2 ? 2 : 4;
+    static_assert(NT % 32 == 0 && (NW & (NW - 1)) == 0 && NW * NP <= 32, "warp sums in one warp");
+    __shared__ V red[NW * NP];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    V v[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) v[k] = k < NV ? in[k < NV ? k : 0] : V{};
+    int m = 16;
+    if constexpr (NP == 4) {
+        const bool hi = lane & m;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) v[k] = sum_of(hi ? v[k + 2] : v[k], shfl_xor_(hi ? v[k] : v[k + 2], m));
+        m >>= 1;
+    }
+    if constexpr (NP >= 2) {
+        const bool hi = lane & m;
+        v[0] = sum_of(hi ? v[1] : v[0], shfl_xor_(hi ? v[0] : v[1], m));
+        m >>= 1;
+    }
+    for (; m > 0; m >>= 1) v[0] = sum_of(v[0], shfl_xor_(v[0], m));
+    // lanes 0, 32 / NP, ... hold the warp's NP sums
+    constexpr int STEP = 32 / NP;
+    if (lane % STEP == 0) red[(lane / STEP) * NW + wid] = v[0];
+    __syncthreads();
+    if (wid == 0) {
+        V r = lane < NW * NP ? red[lane] : V{};
+#pragma unroll
+        for (int q = NW / 2; q > 0; q >>= 1) r = sum_of(r, shfl_xor_(r, q));
+        const double d = as_double(r);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            // value k's lane group: with NP = 4 the first step split (0,1) | (2,3)
+            out[k] = __shfl_sync(0xffffffffu, d, k * NW);
+        }
+    }
+}
 
 constexpr int DG_NT = 256;
 
 // P_B scale of block `blk` (Section 3.3, Eq. "proj-L2" as a radial scale):
-// eps / ||w - y|| if that norm exceeds eps, else 1, from the previous step's
-// chunk partials summed in a fixed order (the same result in every CTA).
-// With `test`, *stop also receives Algorithm 2's stopping test of the
-// previous step, ||zbar^t - zbar^(t-1)|| <= inner_tol ||zbar^t||, in FP64.
-// Every thread of the CTA loads a strided share of the block's contiguous
-// slots (one round trip), then a fixed-order tree and warp order sum them.
-template <typename R> __device__ double block_scale(const VisArgs<R> &A, int blk, bool test = false,
-                                                   bool *stop = nullptr) {
-    __shared__ double sc_s;
-    __shared__ int st_s;
-    __shared__ double red[3][32];
-    double a = 0, dd = 0, nn = 0;
-    for (int k = A.blk_ptr[blk] + threadIdx.x; k < A.blk_ptr[blk + 1]; k += blockDim.x) {
-        const double *q = A.part_in + NPART * (int64_t)k;
-        a += q[0];
+// eps / ||w - y|| if that norm exceeds eps, else 1, from the block's norm
+// partials summed in FP64 in a fixed order.  With `test`, Algorithm 2's
+// stopping test of this step, ||zbar^t - zbar^(t-1)|| <= inner_tol ||zbar^t||,
+// in FP64: a block whose test holds is marked stopped at this step.
+// Run once per block and step, by the CTA that finishes the block's last
+// work unit (unit_done): in the prologue of every CTA of the next kernel it
+// took 18 of the gridding's 46 us at 512^2 with 16 blocks and nearly all of
+// a sub-iteration's 61 us (640 x 480, 12 blocks), as each CTA's FP64 adds
+// queue for the SM's two FP64 lanes.
+template <int NT, typename R> __device__ __forceinline__ void block_scale(const VisArgs<R> &A, int blk, bool test) {
+    double v[3] = {0, 0, 0};
+    const int k1 = A.blk_ptr[blk + 1];
+    for (int k = A.blk_ptr[blk] + threadIdx.x; k < k1; k += NT) {
+        const double *q = A.partials + NPART * (int64_t)k;
+        v[0] += __ldcg(q);
         if (test) {
-            dd += q[2];
-            nn += q[3];
+            v[1] += __ldcg(q + 2);
+            v[2] += __ldcg(q + 3);
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        dd += __shfl_down_sync(0xffffffffu, dd, o);
-        nn += __shfl_down_sync(0xffffffffu, nn, o);
-    }
-    const int wid = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
-        red[0][wid] = a;
-        red[1][wid] = dd;
-        red[2][wid] = nn;
-    }
-    __syncthreads();
+    double t[3];
+    cta_sums<NT, 3, double>(v, t);
     if (threadIdx.x == 0) {
-        double sa = 0, sd = 0, sn = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            sa += red[0][w];
-            sd += red[1][w];
-            sn += red[2][w];
-        }
-        const double nrm = sqrt(sa);
+        const double nrm = sqrt(t[0]);
         if (!isfinite(nrm)) atomicOr(A.err, ERR_NONFINITE);
-        sc_s = (nrm > A.eps[blk]) ? A.eps[blk] / nrm : 1.0;
-        st_s = test && sqrt(sd) <= A.inner_tol * sqrt(sn);
+        A.scale[blk] = (R)((nrm > A.eps[blk]) ? A.eps[blk] / nrm : 1.0);
+        if (test && sqrt(t[1]) <= A.inner_tol * sqrt(t[2])) A.inner_state[blk] = A.step;
     }
     __syncthreads();
-    if (stop) *stop = st_s != 0;
-    return sc_s;
 }
 
-// Step at which block `blk` stopped Algorithm 2 in this iteration (0: still
-// running), read once per CTA so that every thread takes the same branch.
-template <typename R> __device__ int inner_stopped(const VisArgs<R> &A, int blk) {
-    __shared__ int s_state;
-    if (threadIdx.x == 0) s_state = (A.inner_tol > 0) ? *(volatile const int *)(A.inner_state + blk) : 0;
-    __syncthreads();
-    return s_state;
+// Thread 0, after it wrote a unit's partials: counts the unit; true for the
+// block's last one, whose CTA then reads all of the block's partials.
+template <typename R> __device__ __forceinline__ bool unit_done(const VisArgs<R> &A, int blk) {
+    int old;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(A.blk_done + blk) : "memory");
+    return old == A.blk_ptr[blk + 1] - A.blk_ptr[blk] - 1;
 }
 
 // ----------------------------------------------------------------- degrid
@@ -316,7 +345,7 @@ __global__ void __launch_bounds__(NTD, sizeof(R) == 4 ? 768 / NTD : 1)
     };
     uint32_t ph = 0u;   // bit b: parity of the next completion of bar[b]
     const int32_t *ord = A.u_order;
-    __shared__ int claim_s;
+    __shared__ int claim_s, last_s, out_s;
     auto claim = [&](int from) {   // thread 0: the next position after `from` (n_units: none)
         claim_s = from < n_units ? (int)gridDim.x + atomicAdd(A.claim, 1) : n_units;
     };
@@ -366,7 +395,7 @@ __global__ void __launch_bounds__(NTD, sizeof(R) == 4 ? 768 / NTD : 1)
             __syncthreads();
         }
         const int blk = A.ch_block[ch];
-        const double mu = (MODE != DG_OP) ? A.mu[blk] : 0.0;
+        const R mu = (MODE != DG_OP) ? A.mu[blk] : R(0);
         // block outside the active set D: z, w untouched (only the residual
         // statistic is formed); block without a prox output yet: w = z, so
         // that the next Algorithm 2 step starts from P_B(z)
@@ -415,7 +444,7 @@ __global__ void __launch_bounds__(NTD, sizeof(R) == 4 ? 768 / NTD : 1)
                         ww = zz;
                         if (keep_start) A.p[gi] = zz;
                     } else {
-                        const R mu_u = (R)mu * cur.rc.U;
+                        const R mu_u = mu * cur.rc.U;
                         ww = C{cur.p.x - mu_u * (cur.p.x - zz.x), cur.p.y - mu_u * (cur.p.y - zz.y)};
                     }
                     A.w[gi] = ww;
@@ -430,19 +459,39 @@ __global__ void __launch_bounds__(NTD, sizeof(R) == 4 ? 768 / NTD : 1)
         // this thread's first visibility of the next unit (loaded during the
         // unit's reduction and barrier below)
         if (nxt < n_units && (int)threadIdx.x < A.u_count[nxt]) load_vis<R, MODE>(A, A.u_start[nxt] + threadIdx.x, cur);
-        if (MODE != DG_OP) cta_sum2<NTD>(s_w.get(), s_r.get(), A.partials + NPART * (int64_t)A.u_pos[u]);
         // the position after the next unit (read after the barrier below;
         // rewritten only after the next unit's first barrier)
         if (threadIdx.x == 0) claim(nxt_pos);
+        if constexpr (MODE != DG_OP) {
+            const decltype(s_w.get()) part[2] = {s_w.get(), s_r.get()};
+            double sum[2];
+            cta_sums<NTD>(part, sum);
+            if (threadIdx.x == 0) {
+                double *out = A.partials + NPART * (int64_t)A.u_pos[u];
+                out[0] = sum[0];
+                out[1] = sum[1];
+                last_s = unit_done(A, blk);
+            }
+        }
         __syncthreads();   // the tile buffer is refilled two units later
+        if constexpr (MODE != DG_OP) {
+            if (last_s) block_scale<NTD>(A, blk, false);
+        }
     }
     // no claim follows this CTA's exit: the last CTA out resets the counters
+    // (the blocks' too: a launch whose wait ran out leaves units undone)
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(A.claim + 1, 1) == (int)gridDim.x - 1) {
+        out_s = atomicAdd(A.claim + 1, 1) == (int)gridDim.x - 1;
+        if (out_s) {
             A.claim[0] = 0;
             A.claim[1] = 0;
         }
+    }
+    if constexpr (MODE != DG_OP) {
+        __syncthreads();
+        if (out_s)
+            for (int j = threadIdx.x; j < A.n_blocks; j += NTD) A.blk_done[j] = 0;
     }
 }
 
@@ -454,7 +503,7 @@ __global__ void __launch_bounds__(NTD, sizeof(R) == 4 ? 768 / NTD : 1)
 // warm-start array (beta = 0: p_prev is not read; write_p = 0: p not written).
 // only_first: the extra step that moves the start of a block with no prox
 // output yet from z to P_B(z) (randomised active sets); chunks of other
-// blocks, and of blocks outside D, pass their partial through unchanged.
+// blocks, and of blocks outside D, leave their scale as it is.
 // Stopping test (inner_tol > 0): p is kept every step; a step k >= 1 also
 // forms the partials ||p - p_prev||^2 and ||p||^2; a block whose test held
 // for the previous step (or earlier) stops, its p being the prox output.
@@ -466,22 +515,13 @@ __global__ void __launch_bounds__(DG_NT) k_subiter(VisArgs<R> A, int only_first,
     pdl_enter();
     const bool act = !A.bmask || A.bmask[blk];
     const bool first_blk = A.seen && !A.seen[blk];
-    if (!act || (only_first && !first_blk)) {
-        if (threadIdx.x == 0) {
-            const int64_t slot = NPART * (int64_t)A.u_pos[u];
-            A.partials[slot] = A.part_in[slot];
-        }
-        return;
-    }
+    if (!act || (only_first && !first_blk)) return;   // (the same for every unit of the block)
     const bool tol_on = A.inner_tol > 0;
-    if (inner_stopped(A, blk)) return;   // stopped at an earlier step of this iteration
-    bool stop = false;
-    const R c = (R)block_scale(A, blk, tol_on && A.test_in, &stop);
-    if (stop) {   // the previous step's output is the prox
-        if (threadIdx.x == 0) A.inner_state[blk] = A.step - 1;
-        return;
-    }
-    const R mu = (R)A.mu[blk];
+    // stopped at an earlier step of this iteration (this launch's own mark
+    // comes after every unit of the block has finished)
+    if (tol_on && A.inner_state[blk]) return;
+    const R c = A.scale[blk];
+    const R mu = A.mu[blk];
     const bool test_out = tol_on && A.step > 0;
     const bool keep = write_p || tol_on;
     Acc<R> s_w, s_d, s_n;
@@ -507,31 +547,34 @@ __global__ void __launch_bounds__(DG_NT) k_subiter(VisArgs<R> A, int only_first,
         const R dx = wn.x - yy.x, dy = wn.y - yy.y;
         s_w.add(dx * dx + dy * dy);
     }
-    __shared__ double o3[3];
-    cta_sum3<DG_NT>(s_w.get(), s_d.get(), s_n.get(), o3);
+    __shared__ int last_s;
+    const decltype(s_w.get()) part[3] = {s_w.get(), s_d.get(), s_n.get()};
+    double sum[3];
+    cta_sums<DG_NT>(part, sum);
     if (threadIdx.x == 0) {
         double *out = A.partials + NPART * (int64_t)A.u_pos[u];
-        out[0] = o3[0];
-        out[2] = o3[1];
-        out[3] = o3[2];
+        out[0] = sum[0];
+        out[2] = sum[1];
+        out[3] = sum[2];
+        last_s = unit_done(A, blk);
+        if (last_s) A.blk_done[blk] = 0;
     }
+    __syncthreads();
+    if (last_s) block_scale<DG_NT>(A, blk, test_out);
 }
 
 // ----------------------------------------------------------------- block norms
-// One warp per block j: n2 = sum of the block's chunk partials (fixed order),
-// scale_j = eps_j / ||w_j - y_j|| if that norm exceeds eps_j, else 1 (the
-// l2-ball projection P_B of Section 3.3 as a radial scale).
-__global__ void k_block_norms(const double *__restrict__ partials, const int32_t *__restrict__ blk_ptr,
-                              const double *__restrict__ eps, int d,
-                              int with_resid, double *__restrict__ scale, double *__restrict__ resid2,
-                              int *__restrict__ err) {
+// One warp per block j: ||Phi_j xt - y_j||^2 of the last data step from the
+// block's partials (fixed order), for the statistics and the stopping rule.
+__global__ void k_block_norms(const double *__restrict__ partials, const int32_t *__restrict__ blk_ptr, int d,
+                              double *__restrict__ resid2, int *__restrict__ err) {
     const int j = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (j >= d) return;
     double a = 0, b = 0;
     for (int k = blk_ptr[j] + lane; k < blk_ptr[j + 1]; k += 32) {
         a += partials[NPART * (int64_t)k];
-        if (with_resid) b += partials[NPART * (int64_t)k + 1];
+        b += partials[NPART * (int64_t)k + 1];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -539,10 +582,8 @@ __global__ void k_block_norms(const double *__restrict__ partials, const int32_t
         b += __shfl_down_sync(0xffffffffu, b, o);
     }
     if (lane == 0) {
-        const double n = sqrt(a);
-        if (!isfinite(n)) atomicOr(err, ERR_NONFINITE);
-        scale[j] = (n > eps[j]) ? eps[j] / n : 1.0;
-        if (with_resid) resid2[j] = b;
+        if (!isfinite(sqrt(a))) atomicOr(err, ERR_NONFINITE);
+        resid2[j] = b;
     }
 }
 
@@ -596,21 +637,10 @@ __global__ void __launch_bounds__(NW * 32) k_grid(VisArgs<R> A, cplx_t<R> *__res
     // the stopping step kept, not P_B of the current w
     bool done = false;
     if (MODE == GR_DUAL && act) {
-        const bool tol_on = A.inner_tol > 0 && A.n_itr > 1;
-        int steps = A.n_itr;
-        const int stopped = tol_on ? inner_stopped(A, blk) : 0;
-        if (stopped) {
-            done = true;
-            steps = stopped;
-        } else {
-            bool stop = false;
-            c = (R)block_scale(A, blk, tol_on && A.test_in, &stop);
-            if (stop) {
-                done = true;
-                steps = A.n_itr - 1;
-            }
-        }
-        if (threadIdx.x == 0 && A.inner_steps) A.inner_steps[blk] = steps;
+        const int stopped = A.inner_tol > 0 && A.n_itr > 1 ? A.inner_state[blk] : 0;
+        done = stopped != 0;
+        c = A.scale[blk];
+        if (threadIdx.x == 0 && A.inner_steps) A.inner_steps[blk] = done ? stopped : A.n_itr;
     }
     if (MODE == GR_DUAL && act && A.seen && threadIdx.x == 0) A.seen[blk] = 1;
     __syncthreads();
@@ -846,10 +876,11 @@ template <typename R> VisArgs<R> make_args(ppd_ctx *c) {
     A.z = static_cast<cplx_t<R> *>(c->z);
     A.w = static_cast<cplx_t<R> *>(c->w);
     A.p = static_cast<cplx_t<R> *>(c->p);
-    A.mu = c->mu_d;
-    A.scale = c->scale;
-    A.partials = c->part_out;
-    A.part_in = c->part_in;
+    A.mu = static_cast<const R *>(c->mu_d);
+    A.scale = static_cast<R *>(c->scale);
+    A.blk_done = c->blk_done;
+    A.n_blocks = c->d;
+    A.partials = c->partials;
     A.blk_ptr = c->ch.blk_ptr;
     A.u_pos = c->ch.u_pos;
     A.u_start = c->ch.u_start;
@@ -864,7 +895,6 @@ template <typename R> VisArgs<R> make_args(ppd_ctx *c) {
     A.regrid = c->rand_on ? c->regrid_d : nullptr;
     A.inner_tol = c->cfg.inner_tol;
     A.step = c->next_step;
-    A.test_in = c->next_test_in;
     A.n_itr = c->cfg.n_itr;
     A.inner_state = c->inner_state;
     A.inner_steps = c->inner_steps;
@@ -1031,12 +1061,11 @@ template <typename R> int subiter(ppd_ctx *c, cudaStream_t s, int only_first, do
     return launch_end(c, site, s);
 }
 
-int block_norms(ppd_ctx *c, int with_resid, cudaStream_t s) {
+int block_norms(ppd_ctx *c, cudaStream_t s) {
     int site;
     PPD_CHECK(launch_begin(c, "block_norms", s, &site));
     const int wpb = 8;
-    k_block_norms<<<(c->d + wpb - 1) / wpb, wpb * 32, 0, s>>>(c->part_out, c->ch.blk_ptr, c->eps_d,
-                                                               c->d, with_resid, c->scale, c->resid2, c->err);
+    k_block_norms<<<(c->d + wpb - 1) / wpb, wpb * 32, 0, s>>>(c->partials, c->ch.blk_ptr, c->d, c->resid2, c->err);
     return launch_end(c, site, s);
 }
 
