@@ -749,7 +749,7 @@ int ppd_create(ppd_ctx **out, const ppd_config *cfg) {
         (st = dalloc_bytes(&c->twst0, c->K0 * cb)) || (st = dalloc_bytes(&c->twst1, c->K1 * cb)) ||
         (st = dalloc_bytes(&c->deap0, c->L0 * rb)) ||
         (st = dalloc_bytes(&c->deap1, c->L1 * rb)) ||
-        (st = dalloc_bytes(&c->kbpoly, (KB_DEG + 1) * KB_J * sizeof(float))) || (st = dalloc(&c->err, 1)) ||
+        (st = dalloc(&c->err, 1)) ||
         (st = dalloc(&c->stat_out, 3)))
         return bail(st);
     c->n_prim_blocks = (int)std::min<int64_t>((N + 255) / 256, 152 * 4);
@@ -764,7 +764,7 @@ int ppd_create(ppd_ctx **out, const ppd_config *cfg) {
         cudaMemsetAsync(c->blk_seen, 0, (size_t)c->d, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->regrid_d, 0, sizeof(int), c->stream) != cudaSuccess)
         return bail(fail(PPD_ERR_CUDA, "ppd_create: initialisation"));
-    if ((st = make_twiddles(c)) || (st = make_deapodisation(c)) || (st = make_filters(c)) || (st = make_kb_poly(c)))
+    if ((st = make_twiddles(c)) || (st = make_kb_poly(c)) || (st = make_deapodisation(c)) || (st = make_filters(c)))
         return bail(st);
     if (cudaMemsetAsync(c->grid_a, 0, G * cb, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->grid_v, 0, G * cb, c->stream) != cudaSuccess || reset_state(c) != PPD_OK)
@@ -794,7 +794,7 @@ void ppd_destroy(ppd_ctx *c) {
                     (void *)c->dg_claim})
         dfree(p);
     for (void *p : {c->x, c->xt, c->g, c->ut, c->xtrue, c->u, c->wtmp, c->wtmp2, c->grid_a, c->grid_v, c->fft_tmp,
-                    c->tw0, c->tw1, c->twst0, c->twst1, c->deap0, c->deap1, c->kbpoly, (void *)c->prim_part, (void *)c->stat_out,
+                    c->tw0, c->tw1, c->twst0, c->twst1, c->deap0, c->deap1, (void *)c->prim_part, (void *)c->stat_out,
                     (void *)c->err})
         dfree(p);
     if (c->stream2) {

@@ -42,7 +42,6 @@ template <> struct __align__(16) VisRec<float> { int packed; float f0, f1, U; };
 template <> struct __align__(16) VisRec<double> { int packed; int pad; double f0, f1, U; };
 
 constexpr int KB_J = 8;          // interpolation taps per axis
-constexpr int KB_DEG = 7;        // degree of the per-tap FP32 weight polynomial (fit error 4e-8)
 constexpr int HALO = 8;          // extended tile = (T + HALO)^2 cells
 constexpr int N_BASES = 9;       // Dirac + db1..db8
 constexpr int N_WAVELETS = 8;
@@ -184,8 +183,9 @@ struct ppd_ctx {
     ppd::FftPlan plan0, plan1;                                               // FFT plans of K0 (columns), K1 (rows)
     void *twst0 = nullptr, *twst1 = nullptr;   // twiddles of the power-of-two core, stage by stage
     void *filt = nullptr;       // 8 x 16 reals (low-pass, zero padded)
-    void *kbpoly = nullptr;     // (KB_DEG+1) x 8 floats
-    std::vector<float> kbpoly_h;   // host copy (kernel argument of the visibility kernels)
+    std::vector<double> kbpoly_h;   // weight polynomials (kernel argument of the visibility kernels)
+    double kb_inv_i0b = 0;          // 1 / I0(beta)
+    int kb_bessel = 0;              // FP64: the polynomials do not resolve this Kaiser-Bessel shape
     double *prim_part = nullptr;
     int n_prim_blocks = 0;
     int n_stat_parts = 0;        // primal statistics partials the last primal launch wrote

@@ -884,12 +884,13 @@ int make_twiddles(ppd_ctx *c) {
 // Z's scaling s(n) = 1 / psi_hat((n - L/2)/K), psi_hat(f) = (J / I0(beta)) sinh(q)/q,
 // q = sqrt(beta^2 - (pi J f)^2): the Fourier transform of the Kaiser-Bessel kernel.
 static int upload_deapodisation(ppd_ctx *c, int L, int K, void *dst) {
-    const double J = KB_J, beta = c->beta, i0b = std::cyl_bessel_i(0.0, beta);
+    // 1/I0(beta) as the weights have it (make_kb_poly), so that its rounding cancels
+    const double J = KB_J, beta = c->beta, inv_i0b = c->kb_inv_i0b;
     std::vector<double> s(L);
     for (int n = 0; n < L; ++n) {
         double f = ((double)n - L / 2) / (double)K;
         double q = std::sqrt(beta * beta - (M_PI * J * f) * (M_PI * J * f));
-        s[n] = 1.0 / ((J / i0b) * std::sinh(q) / q);
+        s[n] = 1.0 / ((J * inv_i0b) * std::sinh(q) / q);
     }
     if (c->is_f32) {
         std::vector<float> f(s.begin(), s.end());

@@ -16,6 +16,7 @@
 // interior tiles, wrapped plain loads at the grid edge) for degridding, or
 // accumulates into it for gridding.
 #include <cmath>
+#include <limits>
 
 #include "common.cuh"
 #include "tma.cuh"
@@ -74,29 +75,45 @@ __global__ void k_cell_count(const int32_t *__restrict__ cell, const int32_t *__
 }
 
 // ----------------------------------------------------------------- weights
-// FP32: per tap j a degree-KB_DEG polynomial in t = 2 frac - 1 (Chebyshev fit
-// of psi(frac + 3 - j) made on the host); coefficients p[k*8 + j].  p is a
-// kernel argument, so with the loops unrolled every coefficient is a
-// constant-bank operand of its FMA: no load instruction.
-constexpr int KB_NC = (KB_DEG + 1) * KB_J;
-__device__ __forceinline__ void kb_weights(float frac, float (&w)[KB_J], const float (&p)[KB_NC], double, double) {
-    const float t = fmaf(2.0f, frac, -1.0f);
-#pragma unroll
-    for (int j = 0; j < KB_J; ++j) w[j] = p[KB_DEG * KB_J + j];
-#pragma unroll
-    for (int k = KB_DEG - 1; k >= 0; --k)
-#pragma unroll
-        for (int j = 0; j < KB_J; ++j) w[j] = fmaf(w[j], t, p[k * KB_J + j]);
+// Tap j = 0..3 has the weight psi(frac + 3 - j) as a polynomial in t = 2 frac
+// - 1, fitted on the host (make_kb_poly) and evaluated as even + t odd part in
+// t^2; psi is even, so tap 7 - j is the mirror image even - t odd and the pair
+// costs one evaluation (FP32: 32 FMAs an axis instead of 56 for eight Horner
+// chains).  The coefficients p[j KB_N + k] of t^k are kernel arguments, so
+// with the loops unrolled each is a constant-bank operand: no load.
+//
+// FP32: 8 coefficients, fit error 4e-8, below the rounding (8.6e-8 at most,
+// 2.2e-8 rms against 64-bit values; Horner had 8.2e-8, 2.1e-8).
+// FP64: 16 coefficients reach 2.2e-16 at most, 4e-17 rms for the default
+// shape beta = 2.34 J, closer than the Bessel function itself, whose 16
+// evaluations a visibility were most of the FP64 visibility kernels' time on
+// two FP64 lanes per SM.  A shape the 16 coefficients do not resolve (checked
+// on the host) keeps the Bessel function (bessel).
+template <typename R> constexpr int KB_N = sizeof(R) == 4 ? 8 : 16;
+__device__ __noinline__ double kb_bessel(double frac, int j, double beta, double inv_i0b) {
+    const double d = (frac + (double)(3 - j)) * 0.25, x = 1.0 - d * d;
+    return x >= 0.0 ? cyl_bessel_i0(beta * sqrt(x)) * inv_i0b : 0.0;
 }
-
-// FP64: the kernel itself, psi(d) = I0(beta sqrt(1 - (d/4)^2)) / I0(beta), d = frac + 3 - j.
-__device__ __forceinline__ void kb_weights(double frac, double (&w)[KB_J], const float (&)[KB_NC], double beta,
-                                           double inv_i0b) {
+template <typename R, typename A> __device__ __forceinline__ void kb_weights(R frac, R (&w)[KB_J], const A &args) {
+    constexpr int N = KB_N<R>;
+    if constexpr (sizeof(R) == 8) {
+        if (args.bessel) {
 #pragma unroll
-    for (int j = 0; j < KB_J; ++j) {
-        const double dd = (frac + (double)(3 - j)) * 0.25;
-        const double x = 1.0 - dd * dd;
-        w[j] = x >= 0.0 ? cyl_bessel_i0(beta * sqrt(x)) * inv_i0b : 0.0;
+            for (int j = 0; j < KB_J; ++j) w[j] = kb_bessel(frac, j, args.beta, args.inv_i0b);
+            return;
+        }
+    }
+    const R t = fma(R(2), frac, R(-1)), s = t * t;
+#pragma unroll
+    for (int j = 0; j < KB_J / 2; ++j) {
+        R e = args.kbp[j * N + N - 2], o = args.kbp[j * N + N - 1];
+#pragma unroll
+        for (int k = N - 4; k >= 0; k -= 2) {
+            e = fma(e, s, args.kbp[j * N + k]);
+            o = fma(o, s, args.kbp[j * N + k + 1]);
+        }
+        w[j] = fma(o, t, e);
+        w[KB_J - 1 - j] = fma(-o, t, e);
     }
 }
 
@@ -113,7 +130,8 @@ template <typename R> struct VisArgs {
     // [1] CTAs finished (both back to zero after every launch)
     int *claim;
     int K0, K1, ntile1;
-    float kbp[KB_NC];   // the FP32 weight polynomials (kb_weights)
+    R kbp[KB_J / 2 * KB_N<R>];   // the weight polynomials (kb_weights)
+    int bessel;                  // FP64: the weights come from the Bessel function
     double beta, inv_i0b;
     const cplx_t<R> *y;
     cplx_t<R> *v, *z, *w, *p;
@@ -415,8 +433,8 @@ __global__ void __launch_bounds__(NTD, sizeof(R) == 4 ? 768 / NTD : 1)
             if (i + NTD < count) load_vis<R, MODE>(A, gi + NTD, nx);
             const int lb0 = (cur.rc.packed & 0xffff) - row0, lb1 = ((cur.rc.packed >> 16) & 0xffff) - col0;
             R w0[KB_J], w1[KB_J];
-            kb_weights(cur.rc.f0, w0, A.kbp, A.beta, A.inv_i0b);
-            kb_weights(cur.rc.f1, w1, A.kbp, A.beta, A.inv_i0b);
+            kb_weights(cur.rc.f0, w0, A);
+            kb_weights(cur.rc.f1, w1, A);
             C q{0, 0};
 #pragma unroll
             for (int a = 0; a < KB_J; ++a) {
@@ -737,8 +755,8 @@ __global__ void __launch_bounds__(NW * 32) k_grid(VisArgs<R> A, cplx_t<R> *__res
             const R th = cur.th;
             const C tv{th * vv.x, th * vv.y};
             R w0[KB_J], w1[KB_J];
-            kb_weights(rc.f0, w0, A.kbp, A.beta, A.inv_i0b);
-            kb_weights(rc.f1, w1, A.kbp, A.beta, A.inv_i0b);
+            kb_weights(rc.f0, w0, A);
+            kb_weights(rc.f1, w1, A);
 #pragma unroll
             for (int a = 0; a < KB_J / 2; ++a) {   // lane rows (a, a+4) read one pair
                 C *da = sa + 2 * (a * SP + lane);
@@ -868,9 +886,10 @@ template <typename R> VisArgs<R> make_args(ppd_ctx *c) {
     A.K0 = c->K0;
     A.K1 = c->K1;
     A.ntile1 = c->K1 / c->T;
-    for (int i = 0; i < KB_NC; ++i) A.kbp[i] = c->kbpoly_h.empty() ? 0.f : c->kbpoly_h[i];
+    for (int i = 0; i < KB_J / 2 * KB_N<R>; ++i) A.kbp[i] = (R)c->kbpoly_h[i];
+    A.bessel = c->kb_bessel;
     A.beta = c->beta;
-    A.inv_i0b = 1.0 / std::cyl_bessel_i(0.0, c->beta);
+    A.inv_i0b = c->kb_inv_i0b;
     A.y = static_cast<const cplx_t<R> *>(c->y);
     A.v = static_cast<cplx_t<R> *>(c->v);
     A.z = static_cast<cplx_t<R> *>(c->z);
@@ -996,42 +1015,83 @@ int bin_all(ppd_ctx *c, const double *uv_d, const int32_t *blk_d, int64_t M, uin
     return PPD_OK;
 }
 
-// Chebyshev interpolation (degree KB_DEG, in t = 2 frac - 1) of each tap's
-// weight psi(frac + 3 - j), converted to monomial coefficients for Horner.
-int make_kb_poly(ppd_ctx *c) {
-    const int n = KB_DEG + 1;
-    const double beta = c->beta, i0b = std::cyl_bessel_i(0.0, beta);
-    std::vector<float> out((size_t)n * KB_J);
-    for (int j = 0; j < KB_J; ++j) {
-        std::vector<double> fk(n), cheb(n, 0.0);
+// I0(z) by its power series sum_k (z^2/4)^k / (k!)^2 (all terms positive, so
+// the sum is as exact as the type).
+template <typename X> static X bessel_i0(X z) {
+    const X q = z * z / 4;
+    X sum = 1, term = 1;
+    for (int k = 1; k < 100000; ++k) {
+        term *= q / ((X)k * k);
+        sum += term;
+        if (!(term > sum * std::numeric_limits<X>::epsilon() / 4)) break;
+    }
+    return sum;
+}
+
+// Chebyshev interpolation (in t = 2 frac - 1, n points) of the weights
+// psi(frac + 3 - j) of taps 0..3, converted to n monomial coefficients per
+// tap, in type X.
+template <typename X> static std::vector<X> fit_weights(int n, X beta) {
+    const X i0b = bessel_i0<X>(beta), pi = std::acos((X)-1);
+    std::vector<X> out((size_t)n * KB_J / 2), node(n), cs((size_t)n * n);
+    for (int k = 0; k < n; ++k) {
+        node[k] = std::cos(pi * (k + (X)0.5) / n);
+        for (int m = 0; m < n; ++m) cs[(size_t)m * n + k] = std::cos(pi * ((m * (2 * k + 1)) % (4 * n)) / (2 * n));
+    }
+    for (int j = 0; j < KB_J / 2; ++j) {
+        std::vector<X> fk(n), cheb(n, 0), mono(n, 0), Tm1(n, 0), Tm(n, 0), Tn(n, 0);
         for (int k = 0; k < n; ++k) {
-            const double t = std::cos(M_PI * (k + 0.5) / n);
-            const double d = (t + 1.0) * 0.5 + 3.0 - j;
-            const double x = 1.0 - (d / 4.0) * (d / 4.0);
-            fk[k] = x >= 0 ? std::cyl_bessel_i(0.0, beta * std::sqrt(x)) / i0b : 0.0;
+            const X d = ((node[k] + 1) / 2 + 3 - j) / 4;
+            fk[k] = bessel_i0<X>(beta * std::sqrt(1 - d * d)) / i0b;   // |d| < 1 at every node
         }
         for (int m = 0; m < n; ++m) {
-            double s = 0;
-            for (int k = 0; k < n; ++k) s += fk[k] * std::cos(M_PI * m * (k + 0.5) / n);
-            cheb[m] = s * (m == 0 ? 1.0 : 2.0) / n;
+            X s = 0;
+            for (int k = 0; k < n; ++k) s += fk[k] * cs[(size_t)m * n + k];
+            cheb[m] = s * (m == 0 ? 1 : 2) / n;
         }
         // Chebyshev -> monomial: T_0 = 1, T_1 = t, T_{m+1} = 2 t T_m - T_{m-1}
-        std::vector<double> mono(n, 0.0), Tm1(n, 0.0), Tm(n, 0.0), Tn(n, 0.0);
-        Tm1[0] = 1.0;
-        Tm[1] = 1.0;
-        for (int k = 0; k < n; ++k) mono[k] += cheb[0] * Tm1[k];
-        if (n > 1)
-            for (int k = 0; k < n; ++k) mono[k] += cheb[1] * Tm[k];
+        Tm1[0] = 1;
+        Tm[1] = 1;
+        for (int k = 0; k < n; ++k) mono[k] = cheb[0] * Tm1[k] + cheb[1] * Tm[k];
         for (int m = 2; m < n; ++m) {
-            for (int k = 0; k < n; ++k) Tn[k] = (k > 0 ? 2.0 * Tm[k - 1] : 0.0) - Tm1[k];
+            for (int k = 0; k < n; ++k) Tn[k] = (k > 0 ? 2 * Tm[k - 1] : 0) - Tm1[k];
             for (int k = 0; k < n; ++k) mono[k] += cheb[m] * Tn[k];
             Tm1 = Tm;
             Tm = Tn;
         }
-        for (int k = 0; k < n; ++k) out[(size_t)k * KB_J + j] = (float)mono[k];
+        for (int k = 0; k < n; ++k) out[(size_t)j * n + k] = mono[k];
     }
-    PPD_CUDA(cudaMemcpy(c->kbpoly, out.data(), out.size() * sizeof(float), cudaMemcpyHostToDevice));
-    c->kbpoly_h = out;
+    return out;
+}
+
+// The weight polynomials (KB_N coefficients per tap) and 1 / I0(beta).  The
+// FP64 fit runs in long double, so that its coefficients carry only their
+// own rounding (a fit in double leaves 3e-15).  FP64: where the polynomials
+// are off by more than 1e-15 (a shape far from the default) the kernels keep
+// the Bessel function.
+int make_kb_poly(ppd_ctx *c) {
+    c->kb_bessel = 0;
+    if (c->is_f32) {
+        c->kbpoly_h = fit_weights<double>(KB_N<float>, c->beta);
+        c->kb_inv_i0b = 1.0 / bessel_i0<double>(c->beta);
+        return PPD_OK;
+    }
+    using X = long double;
+    const int n = KB_N<double>;
+    const X beta = c->beta, i0b = bessel_i0<X>(beta);
+    const std::vector<X> fit = fit_weights<X>(n, beta);
+    c->kbpoly_h.assign(fit.begin(), fit.end());
+    c->kb_inv_i0b = (double)(1 / i0b);
+    for (int j = 0; j < KB_J / 2; ++j)
+        for (int i = 0; i <= 8; ++i) {
+            const double t = i / 4.0 - 1.0;
+            double v = 0;
+            for (int k = n - 1; k >= 0; --k) v = std::fma(v, t, c->kbpoly_h[(size_t)j * n + k]);
+            const X d = (((X)t + 1) / 2 + 3 - j) / 4, x = 1 - d * d;
+            const X ref = x >= 0 ? bessel_i0<X>(beta * std::sqrt(x)) / i0b : (X)0;
+            // (written so that a value that is not finite also counts)
+            if (!(std::abs((X)v - ref) <= (X)1e-15)) c->kb_bessel = 1;
+        }
     return PPD_OK;
 }
 
