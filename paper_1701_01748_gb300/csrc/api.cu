@@ -124,8 +124,8 @@ void free_vis(ppd_ctx *c) {
     for (void *p : {c->rec, c->theta_v, c->y, c->v, c->z, c->w, c->p, c->y_raw, (void *)c->perm,
                     (void *)c->count_cell, (void *)c->ch.start, (void *)c->ch.count, (void *)c->ch.tile,
                     (void *)c->ch.block, (void *)c->ch.tile_first, (void *)c->ch.tile_n, (void *)c->ch.blk_ptr,
-                    (void *)c->ch.u_start, (void *)c->ch.u_count, (void *)c->ch.u_chunk, (void *)c->ch.u_pos, (void *)c->ch.u_order, (void *)c->ch.order, (void *)c->ch.active, (void *)c->partials, c->scale, (void *)c->resid2,
-                    (void *)c->eps_d, c->mu_d, (void *)c->blk_done, c->gpart})
+                    (void *)c->ch.grp, (void *)c->ch.warp_grp, (void *)c->ch.warp_run, (void *)c->ch.run_pos, (void *)c->ch.order, (void *)c->ch.active, (void *)c->partials, c->scale, (void *)c->resid2,
+                    (void *)c->eps_d, c->mu_d, c->gpart})
         dfree(p);
     c->rec = c->theta_v = c->y = c->v = c->z = c->w = c->p = c->y_raw = c->gpart = nullptr;
     c->perm = nullptr;
@@ -133,7 +133,6 @@ void free_vis(ppd_ctx *c) {
     c->ch = Chunks{};
     c->partials = c->resid2 = c->eps_d = nullptr;
     c->scale = c->mu_d = nullptr;
-    c->blk_done = nullptr;
     c->have_vis = c->have_weights = false;
     c->gpart_stale = true;
 }
@@ -226,7 +225,7 @@ int stop_rule(ppd_ctx *c, double tol, double fac, int *flag) {
 // xt and u, so in the FP32 path it runs on a second stream beside the data
 // branch (FFT, degridding with the data step, gridding, inverse FFT); both
 // join before the primal step.  The per-block P_B scales are computed by
-// the kernel that forms the norms, in the CTA that finishes a block.
+// a small kernel after the one that forms the norms.
 template <typename R> int iteration_body(ppd_ctx *c, cudaStream_t s, bool first) {
     using C = cplx_t<R>;
     C *ga = static_cast<C *>(c->grid_a), *gv = static_cast<C *>(c->grid_v);
@@ -529,7 +528,6 @@ int reset_state(ppd_ctx *c) {
         PPD_CUDA(cudaMemsetAsync(c->p, 0, 2 * c->M * rb, c->stream));
     }
     PPD_CUDA(cudaMemsetAsync(c->err, 0, sizeof(int), c->stream));
-    if (c->blk_done) PPD_CUDA(cudaMemsetAsync(c->blk_done, 0, c->d * sizeof(int), c->stream));
     if (c->blk_seen) PPD_CUDA(cudaMemsetAsync(c->blk_seen, 0, c->d, c->stream));
     if (c->inner_state) PPD_CUDA(cudaMemsetAsync(c->inner_state, 0, c->d * sizeof(int), c->stream));
     if (c->inner_steps) PPD_CUDA(cudaMemsetAsync(c->inner_steps, 0, c->d * sizeof(int), c->stream));
@@ -756,11 +754,9 @@ int ppd_create(ppd_ctx **out, const ppd_config *cfg) {
     if ((st = dalloc(&c->prim_part, 3 * (size_t)std::max(c->n_prim_blocks, c->L0)))) return bail(st);
     if ((st = dalloc(&c->mask_cur, (size_t)c->d + N_BASES)) || (st = dalloc(&c->blk_seen, (size_t)c->d)) ||
         (st = dalloc(&c->regrid_d, 1)) || (st = dalloc(&c->inner_state, (size_t)c->d)) ||
-        (st = dalloc(&c->inner_steps, (size_t)c->d)) || (st = dalloc(&c->stop_flag, 1)) ||
-        (st = dalloc(&c->dg_claim, 2)))
+        (st = dalloc(&c->inner_steps, (size_t)c->d)) || (st = dalloc(&c->stop_flag, 1)))
         return bail(st);
     if (cudaMemsetAsync(c->mask_cur, 1, (size_t)c->d + N_BASES, c->stream) != cudaSuccess ||
-        cudaMemsetAsync(c->dg_claim, 0, 2 * sizeof(int), c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->blk_seen, 0, (size_t)c->d, c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->regrid_d, 0, sizeof(int), c->stream) != cudaSuccess)
         return bail(fail(PPD_ERR_CUDA, "ppd_create: initialisation"));
@@ -790,8 +786,7 @@ void ppd_destroy(ppd_ctx *c) {
                     (void *)c->col_fwd, c->fft_tmp_inv})
         dfree(p);
     for (void *p : {c->wgt, c->wcoef, (void *)c->mask_all, (void *)c->mask_cur, (void *)c->blk_seen,
-                    (void *)c->regrid_d, (void *)c->inner_state, (void *)c->inner_steps, (void *)c->stop_flag,
-                    (void *)c->dg_claim})
+                    (void *)c->regrid_d, (void *)c->inner_state, (void *)c->inner_steps, (void *)c->stop_flag})
         dfree(p);
     for (void *p : {c->x, c->xt, c->g, c->ut, c->xtrue, c->u, c->wtmp, c->wtmp2, c->grid_a, c->grid_v, c->fft_tmp,
                     c->tw0, c->tw1, c->twst0, c->twst1, c->deap0, c->deap1, (void *)c->prim_part, (void *)c->stat_out,
@@ -883,6 +878,7 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     const uint64_t KK = (uint64_t)c->K0 * c->K1;
     const int ntiles = (c->K0 / c->T) * (c->K1 / c->T);
     std::vector<int32_t> cs, cn, ct, cbk, tfirst(ntiles, 0), tn(ntiles, 0);
+    std::vector<int4> grp;   // groups of the degridding and sub-iterations
     for (int64_t i = 0; i < M;) {
         const uint64_t k0 = key[c->perm_h[i]];
         const uint64_t tb = k0 / KK;   // tile * d + block
@@ -897,6 +893,9 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
             ct.push_back(tile);
             cbk.push_back(blk);
         }
+        for (int64_t s = i; s < j; s += 32)
+            grp.push_back(make_int4((int)s, (int)std::min<int64_t>(32, j - s), (int)(tb / (uint64_t)c->d),
+                                    (int)(tb % (uint64_t)c->d)));
         i = j;
     }
     const int64_t nch = (int64_t)cs.size();
@@ -936,39 +935,58 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
             }
         }
     }
-    // work units of the degridding and sub-iterations (runs of at most UNIT
-    // visibilities of one chunk) and their block-major partial slots: block
-    // b owns slots bptr[b] .. bptr[b+1] - 1, unit u writes slot upos[u]
-    std::vector<int32_t> us, un, uc;
-    for (int64_t k = 0; k < nch; ++k)
-        for (int32_t o = 0; o < cn[k]; o += UNIT) {
-            us.push_back(cs[k] + o);
-            un.push_back(std::min<int32_t>(UNIT, cn[k] - o));
-            uc.push_back((int32_t)k);
+    // shares of the groups (a share per resident warp of the degridding),
+    // their runs of one block, and the runs' block-major partial slots: block
+    // b owns slots bptr[b] .. bptr[b+1] - 1, run r writes slot rpos[r].
+    // Groups in sparse tiles (few visibilities, a tile copy each) take longer
+    // than those of the dense centre, so a share is `rounds` pieces spread
+    // over the whole order, up to 4 of four groups or more (25 iterations at
+    // 1024^2: 11.05 ms with one piece, 10.96 with up to four; every piece
+    // ends a run, and eight made the degridding 11 % longer in instructions)
+    const int64_t ng = (int64_t)grp.size();
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    const int64_t nwarps = std::min<int64_t>(ng, (int64_t)std::max(sms, 1) * degrid_warps_per_sm(c));
+    const int64_t rounds = std::max<int64_t>(1, std::min<int64_t>(4, ng / (4 * nwarps)));
+    std::vector<int32_t> wgrp(nwarps + 1, 0), wrun(nwarps + 1, 0), rblk;
+    {
+        std::vector<int4> share;
+        share.reserve(ng);
+        for (int64_t w = 0; w < nwarps; ++w) {
+            wgrp[w] = (int32_t)share.size();
+            wrun[w] = (int32_t)rblk.size();
+            for (int64_t r = 0; r < rounds; ++r) {
+                const int64_t k = r * nwarps + w, n = rounds * nwarps;
+                for (int64_t g = k * ng / n; g < (k + 1) * ng / n; ++g) {
+                    if ((int64_t)share.size() == wgrp[w] || grp[g].w != share.back().w) rblk.push_back(grp[g].w);
+                    share.push_back(grp[g]);
+                }
+            }
         }
-    const int64_t nu = (int64_t)us.size();
-    std::vector<int32_t> uord(nu);
-    for (int64_t u = 0; u < nu; ++u) uord[u] = (int32_t)u;
-    std::stable_sort(uord.begin(), uord.end(), [&](int32_t a, int32_t b) { return un[a] > un[b]; });
+        wgrp[nwarps] = (int32_t)share.size();
+        wrun[nwarps] = (int32_t)rblk.size();
+        grp.swap(share);
+    }
+    const int64_t nruns = (int64_t)rblk.size();
+    std::vector<int32_t> bptr(c->d + 1, 0), rpos(nruns);
+    for (int32_t b : rblk) bptr[b + 1]++;
+    for (int j = 0; j < c->d; ++j) bptr[j + 1] += bptr[j];
+    {
+        std::vector<int32_t> fill(bptr.begin(), bptr.end() - 1);
+        for (int64_t r = 0; r < nruns; ++r) rpos[r] = fill[rblk[r]]++;
+    }
     // the gridding's CTA order: chunks by decreasing size
     std::vector<int32_t> cord(nch);
     for (int64_t k = 0; k < nch; ++k) cord[k] = (int32_t)k;
     std::stable_sort(cord.begin(), cord.end(), [&](int32_t a, int32_t b) { return cn[a] > cn[b]; });
-    std::vector<int32_t> bptr(c->d + 1, 0), upos(nu);
-    for (int64_t u = 0; u < nu; ++u) bptr[cbk[uc[u]] + 1]++;
-    for (int j = 0; j < c->d; ++j) bptr[j + 1] += bptr[j];
-    {
-        std::vector<int32_t> fill(bptr.begin(), bptr.end() - 1);
-        for (int64_t u = 0; u < nu; ++u) upos[u] = fill[cbk[uc[u]]]++;
-    }
     c->ch.n = nch;
-    c->ch.nu = nu;
+    c->ch.n_grp = (int32_t)ng;
+    c->ch.n_warps = (int32_t)nwarps;
+    c->ch.n_runs = nruns;
     // default gridding CTA shape (unless configured or autotuned): eight
     // warps while the chunks make few waves, four (more CTAs per SM) beyond
     // twelve chunks per SM
     if (c->cfg.grid_warps == 0 && !c->shape_tuned && c->is_f32) {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
         c->grid_nw = nch > 12LL * std::max(sms, 1) ? 4 : 8;
     }
     c->ch.n_active = (int64_t)active.size();
@@ -977,11 +995,12 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     if ((st = dalloc(&c->ch.start, nch)) || (st = dalloc(&c->ch.count, nch)) || (st = dalloc(&c->ch.tile, nch)) ||
         (st = dalloc(&c->ch.block, nch)) || (st = dalloc(&c->ch.tile_first, ntiles)) ||
         (st = dalloc(&c->ch.tile_n, ntiles)) || (st = dalloc(&c->ch.blk_ptr, c->d + 1)) ||
-        (st = dalloc(&c->ch.u_start, nu)) ||
-        (st = dalloc(&c->ch.u_count, nu)) || (st = dalloc(&c->ch.u_chunk, nu)) || (st = dalloc(&c->ch.u_pos, nu)) || (st = dalloc(&c->ch.u_order, nu)) || (st = dalloc(&c->ch.order, nch)) ||
+        (st = dalloc(&c->ch.grp, ng)) || (st = dalloc(&c->ch.warp_grp, nwarps + 1)) || (st = dalloc(&c->ch.warp_run, nwarps + 1)) ||
+        (st = dalloc(&c->ch.run_pos, nruns)) ||
+        (st = dalloc(&c->ch.order, nch)) ||
         (st = dalloc(&c->ch.active, active.size())) ||
-        (st = dalloc(&c->partials, NPART * (size_t)nu)) ||
-        (st = dalloc_bytes(&c->scale, c->d * c->rsz)) || (st = dalloc(&c->blk_done, c->d)) || (st = dalloc(&c->resid2, c->d)) || (st = dalloc(&c->eps_d, c->d)) ||
+        (st = dalloc(&c->partials, NPART * (size_t)nruns)) ||
+        (st = dalloc_bytes(&c->scale, c->d * c->rsz)) || (st = dalloc(&c->resid2, c->d)) || (st = dalloc(&c->eps_d, c->d)) ||
         (st = dalloc_bytes(&c->mu_d, c->d * c->rsz)) || (st = dalloc_bytes(&c->gpart, (size_t)nch * E * E * cbsz)) ||
         (st = dalloc(&c->perm, M)) || (st = dalloc_bytes(&c->rec, M * (c->is_f32 ? 16 : 32))) ||
         (st = dalloc_bytes(&c->y, M * cbsz)) || (st = dalloc_bytes(&c->v, M * cbsz)) ||
@@ -1013,11 +1032,10 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
         (e = cudaMemcpy(c->ch.tile_first, tfirst.data(), ntiles * 4, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(c->ch.tile_n, tn.data(), ntiles * 4, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(c->ch.blk_ptr, bptr.data(), (c->d + 1) * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->ch.u_start, us.data(), nu * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->ch.u_count, un.data(), nu * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->ch.u_chunk, uc.data(), nu * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->ch.u_pos, upos.data(), nu * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->ch.u_order, uord.data(), nu * 4, cudaMemcpyHostToDevice)) ||
+        (e = cudaMemcpy(c->ch.grp, grp.data(), ng * sizeof(int4), cudaMemcpyHostToDevice)) ||
+        (e = cudaMemcpy(c->ch.warp_grp, wgrp.data(), (nwarps + 1) * 4, cudaMemcpyHostToDevice)) ||
+        (e = cudaMemcpy(c->ch.warp_run, wrun.data(), (nwarps + 1) * 4, cudaMemcpyHostToDevice)) ||
+        (e = cudaMemcpy(c->ch.run_pos, rpos.data(), nruns * 4, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(c->ch.order, cord.data(), nch * 4, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(c->ch.active, active.data(), active.size() * 4, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(c->perm, c->perm_h.data(), M * 8, cudaMemcpyHostToDevice)) ||

@@ -49,7 +49,6 @@ constexpr int MAX_TAPS = 16;     // db8
 // per-chunk norm partials: ||w-y||^2, ||Theta q - y||^2 and, for the
 // Algorithm 2 stopping test, ||zbar^t - zbar^(t-1)||^2, ||zbar^t||^2
 constexpr int NPART = 4;
-constexpr int UNIT = 1 << 30;    // visibilities per work unit of the degridding / sub-iterations (no split: a unit is a chunk)
 constexpr double INV_TWO_PI = 0.15915494309189535;
 
 // device error word bits
@@ -140,13 +139,16 @@ struct Chunks {
     int64_t n = 0;
     int32_t *start = nullptr, *count = nullptr, *tile = nullptr, *block = nullptr;   // device
     int32_t *tile_first = nullptr, *tile_n = nullptr;                                // device, n_tiles
-    // work units of the degridding and sub-iterations: runs of at most UNIT
-    // visibilities of one chunk (device arrays of nu entries); unit u writes
-    // its norm partials to slot u_pos[u], block b owns slots blk_ptr[b] ..
-    // blk_ptr[b+1] - 1; u_order lists the units by decreasing size (the
-    // degridding's visiting order)
-    int64_t nu = 0;
-    int32_t *u_start = nullptr, *u_count = nullptr, *u_chunk = nullptr, *u_pos = nullptr, *u_order = nullptr;
+    // work of the degridding and sub-iterations: groups of at most 32
+    // visibilities of one tile and block {start, count, tile, block}, shared
+    // out equally to n_warps warps (warp w: warp_grp[w] .. warp_grp[w+1] - 1); a warp's maximal sequences
+    // of groups of one block are its runs (warp w: warp_run[w] ..
+    // warp_run[w+1] - 1); run r writes its norm partials to slot
+    // run_pos[r], block b owns slots blk_ptr[b] .. blk_ptr[b+1] - 1
+    int32_t n_grp = 0, n_warps = 0;
+    int64_t n_runs = 0;
+    int4 *grp = nullptr;
+    int32_t *warp_grp = nullptr, *warp_run = nullptr, *run_pos = nullptr;
     int32_t *blk_ptr = nullptr;
     int32_t *order = nullptr;    // chunks by decreasing size (the gridding's CTA order)
     int32_t *active = nullptr;   // tiles the combine pass writes (device)
@@ -210,7 +212,6 @@ struct ppd_ctx {
     ppd::Chunks ch;
     double *partials = nullptr, *resid2 = nullptr, *eps_d = nullptr;
     void *scale = nullptr, *mu_d = nullptr;           // per block, reals: P_B scale of the last step, mu
-    int *blk_done = nullptr;                          // per block: finished work units (zero between launches)
     // Algorithm 2 stopping test (cfg.inner_tol > 0): per block the step at
     // which the test held in the current iteration (0 = still running) and
     // the steps taken in the last iteration; the step number of the next
@@ -218,7 +219,6 @@ struct ppd_ctx {
     int *inner_state = nullptr, *inner_steps = nullptr;
     int next_step = 0;
     int *stop_flag = nullptr;                          // global stopping rule (device, 1 int)
-    int *dg_claim = nullptr;                           // degridding work counters (device, 2 ints, zero between launches)
     cudaStream_t stream2 = nullptr;                   // prior (SARA) branch of the iteration
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     void *gpart = nullptr;           // n_chunks x (T+HALO)^2 complex
@@ -315,6 +315,9 @@ int make_deapodisation(ppd_ctx *c);
 int bin_all(ppd_ctx *c, const double *uv_d, const int32_t *blk_d, int64_t M, uint64_t *key_d, int32_t *base_d,
             double *frac_d, int32_t *count_d, int *bad_d);
 int make_kb_poly(ppd_ctx *c);
+
+// resident degridding warps per SM (the groups are shared out to that many)
+int degrid_warps_per_sm(const ppd_ctx *c);
 
 enum DegridMode { DG_OP = 0, DG_DUAL = 1, DG_FIRST = 2 };
 enum GridMode { GR_OP = 0, GR_OP_U = 1, GR_DUAL = 2 };

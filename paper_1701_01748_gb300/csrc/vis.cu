@@ -123,12 +123,13 @@ template <typename R> struct VisArgs {
     R theta_s;
     const int32_t *ch_start, *ch_count, *ch_tile, *ch_block;
     const int32_t *ch_order;   // chunks by decreasing size: the gridding's CTA order
-    // work units of the degridding and sub-iteration kernels: runs of at
-    // most DG_NT visibilities of one chunk, each with its partial slot
-    const int32_t *u_start, *u_count, *u_chunk, *u_order;
-    // the degridding's work counters: [0] next position in u_order to claim,
-    // [1] CTAs finished (both back to zero after every launch)
-    int *claim;
+    // groups of at most 32 visibilities of one tile and block {start, count,
+    // tile, block}: warp w of the degridding and sub-iteration kernels owns
+    // groups warp_grp[w] .. warp_grp[w + 1] - 1; its maximal sequences of
+    // groups of one block are runs warp_run[w] .. warp_run[w + 1] - 1
+    const int4 *grp;
+    const int32_t *warp_grp, *warp_run;
+    int n_warps;
     int K0, K1, ntile1;
     R kbp[KB_J / 2 * KB_N<R>];   // the weight polynomials (kb_weights)
     int bessel;                  // FP64: the weights come from the Bessel function
@@ -136,12 +137,11 @@ template <typename R> struct VisArgs {
     const cplx_t<R> *y;
     cplx_t<R> *v, *z, *w, *p;
     const R *mu;
-    R *scale;                    // per block: the P_B scale of the last step (block_scale)
-    int *blk_done;               // per block: units of the running launch that are done (zero between launches)
-    double *partials;            // norm partials of the work units
-    // partials live in block-major slots: work unit u writes slot
-    // u_pos[u]; block b's slots are blk_ptr[b] .. blk_ptr[b+1] - 1
-    const int32_t *blk_ptr, *u_pos;
+    const R *scale;              // per block: the P_B scale of the last step (k_block_scale)
+    double *partials;            // norm partials of the runs
+    // partials live in block-major slots: run r writes slot run_pos[r];
+    // block b's slots are blk_ptr[b] .. blk_ptr[b+1] - 1
+    const int32_t *blk_ptr, *run_pos;
     const double *eps;
     int *err;
     // randomised active sets (null: every block active): the current
@@ -159,7 +159,7 @@ template <typename R> struct VisArgs {
     // n_itr: the gridding), per block the step at which the test held (0:
     // running) and the steps taken
     double inner_tol;
-    int step, n_itr, n_blocks;
+    int step, n_itr;
     int *inner_state, *inner_steps;
 };
 
@@ -206,17 +206,14 @@ template <typename R> struct Acc {
     }
 };
 
-// Deterministic CTA sums of NV <= 4 values per thread.  The first shuffle
+// Warp sums of NV <= 4 values per lane (fixed order).  The first shuffle
 // steps also halve the number of values a lane carries (lanes whose bit is
 // set take the upper half), so that NV = 2 costs 5 adds a lane instead of
-// 10; then the warps' sums in a fixed tree.  The sums are valid in thread 0
-// after the call (out[k]); the CTA must pass a barrier before `red` is used
-// again by another call.
-template <int NT, int NV, typename V> __device__ __forceinline__ void cta_sums(const V (&in)[NV], double (&out)[NV]) {
-    constexpr int NW = NT / 32, NP = NV <= 1 ? 1 : NV <= 2 ? 2 : 4;
-    static_assert(NT % 32 == 0 && (NW & (NW - 1)) == 0 && NW * NP <= 32, "warp sums in one warp");
-    __shared__ V red[NW * NP];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+// 10.  Lane k * warp_sum_step(NV) returns the sum of value k.
+__host__ __device__ constexpr int warp_sum_step(int nv) { return nv <= 1 ? 32 : nv <= 2 ? 16 : 8; }
+template <int NV, typename V> __device__ __forceinline__ V warp_sums(const V (&in)[NV]) {
+    constexpr int NP = 32 / warp_sum_step(NV);
+    const int lane = threadIdx.x & 31;
     V v[NP];
 #pragma unroll
     for (int k = 0; k < NP; ++k) v[k] = k < NV ? in[k < NV ? k : 0] : V{};
@@ -233,82 +230,86 @@ template <int NT, int NV, typename V> __device__ __forceinline__ void cta_sums(c
         m >>= 1;
     }
     for (; m > 0; m >>= 1) v[0] = sum_of(v[0], shfl_xor_(v[0], m));
-    // lanes 0, 32 / NP, ... hold the warp's NP sums
-    constexpr int STEP = 32 / NP;
-    if (lane % STEP == 0) red[(lane / STEP) * NW + wid] = v[0];
-    __syncthreads();
-    if (wid == 0) {
-        V r = lane < NW * NP ? red[lane] : V{};
-#pragma unroll
-        for (int q = NW / 2; q > 0; q >>= 1) r = sum_of(r, shfl_xor_(r, q));
-        const double d = as_double(r);
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            // value k's lane group: with NP = 4 the first step split (0,1) | (2,3)
-            out[k] = __shfl_sync(0xffffffffu, d, k * NW);
-        }
-    }
+    return v[0];
 }
 
-constexpr int DG_NT = 256;
 
-// P_B scale of block `blk` (Section 3.3, Eq. "proj-L2" as a radial scale):
-// eps / ||w - y|| if that norm exceeds eps, else 1, from the block's norm
-// partials summed in FP64 in a fixed order.  With `test`, Algorithm 2's
-// stopping test of this step, ||zbar^t - zbar^(t-1)|| <= inner_tol ||zbar^t||,
-// in FP64: a block whose test holds is marked stopped at this step.
-// Run once per block and step, by the CTA that finishes the block's last
-// work unit (unit_done): in the prologue of every CTA of the next kernel it
-// took 18 of the gridding's 46 us at 512^2 with 16 blocks and nearly all of
-// a sub-iteration's 61 us (640 x 480, 12 blocks), as each CTA's FP64 adds
-// queue for the SM's two FP64 lanes.
-template <int NT, typename R> __device__ __forceinline__ void block_scale(const VisArgs<R> &A, int blk, bool test) {
-    double v[3] = {0, 0, 0};
-    const int k1 = A.blk_ptr[blk + 1];
-    for (int k = A.blk_ptr[blk] + threadIdx.x; k < k1; k += NT) {
-        const double *q = A.partials + NPART * (int64_t)k;
-        v[0] += __ldcg(q);
-        if (test) {
-            v[1] += __ldcg(q + 2);
-            v[2] += __ldcg(q + 3);
-        }
-    }
-    double t[3];
-    cta_sums<NT, 3, double>(v, t);
-    if (threadIdx.x == 0) {
-        const double nrm = sqrt(t[0]);
-        if (!isfinite(nrm)) atomicOr(A.err, ERR_NONFINITE);
-        A.scale[blk] = (R)((nrm > A.eps[blk]) ? A.eps[blk] / nrm : 1.0);
-        if (test && sqrt(t[1]) <= A.inner_tol * sqrt(t[2])) A.inner_state[blk] = A.step;
-    }
-    __syncthreads();
+// a w + c on both components: one instruction on packed pairs in FP32 (the
+// same two roundings as two fmaf), half the issue slots of the taps' sums
+struct F32x2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F32x2 pack2(float x, float y) {
+    F32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(F32x2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ F32x2 fma2(F32x2 a, F32x2 b, F32x2 c) {
+    F32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
 }
 
-// Thread 0, after it wrote a unit's partials: counts the unit; true for the
-// block's last one, whose CTA then reads all of the block's partials.
-template <typename R> __device__ __forceinline__ bool unit_done(const VisArgs<R> &A, int blk) {
-    int old;
-    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(A.blk_done + blk) : "memory");
-    return old == A.blk_ptr[blk + 1] - A.blk_ptr[blk] - 1;
+// sum_ab w0[a] w1[b] tile[a][b] over an 8 x 8 footprint, row by row
+template <int E> __device__ __forceinline__ float2 footprint(const float2 *cell, const float (&w0)[KB_J], const float (&w1)[KB_J]) {
+    F32x2 d1[KB_J], q = pack2(0.f, 0.f);
+#pragma unroll
+    for (int b = 0; b < KB_J; ++b) d1[b] = pack2(w1[b], w1[b]);
+#pragma unroll
+    for (int a = 0; a < KB_J; ++a) {
+        const F32x2 *row = reinterpret_cast<const F32x2 *>(cell + a * E);
+        F32x2 r = pack2(0.f, 0.f);
+#pragma unroll
+        for (int b = 0; b < KB_J; ++b) r = fma2(d1[b], row[b], r);
+        q = fma2(pack2(w0[a], w0[a]), r, q);
+    }
+    return unpack2(q);
+}
+template <int E> __device__ __forceinline__ double2 footprint(const double2 *cell, const double (&w0)[KB_J], const double (&w1)[KB_J]) {
+    double2 q{0, 0};
+#pragma unroll
+    for (int a = 0; a < KB_J; ++a) {
+        const double2 *row = cell + a * E;
+        double2 r{0, 0};
+#pragma unroll
+        for (int b = 0; b < KB_J; ++b) {
+            const double2 g = row[b];
+            r.x += w1[b] * g.x;
+            r.y += w1[b] * g.y;
+        }
+        q.x += w0[a] * r.x;
+        q.y += w0[a] * r.y;
+    }
+    return q;
 }
 
 // ----------------------------------------------------------------- degrid
 // mode DG_OP:    op_out[perm[i]] = Theta G a
 // mode DG_DUAL:  z = v/U + Theta G a;  w = p - mu U (p - z)
 // mode DG_FIRST: z = v/U + Theta G a;  w = z   (Algorithm 2 then starts from P_B(z))
-// partial slot of the unit = (||w - y||^2, ||Theta G a - y||^2)
+// partials of a run = (||w - y||^2, ||Theta G a - y||^2)
 //
-// Persistent CTAs walk the work units (the chunks) in the order u_order
-// (largest first): CTA b starts at position b, then every CTA claims its
-// next position from a counter when it starts a unit (so the light units
-// of the tail go to whichever CTAs finish first); the last CTA to finish
-// resets the counters for the next launch.  Which CTA computes a unit does
-// not change any result.
-// The (T+8)^2 grid tile of the next unit is fetched by TMA into the other of
-// two shared buffers while the current unit is computed (interior tiles;
-// tiles that wrap around the grid edge are loaded with plain loads when they
-// are used); each thread loads its first visibility of the next unit before
-// the current one is computed, and one visibility ahead inside a unit.
+// A warp works alone: it owns an equal share of the groups of 32
+// visibilities (a lane each; a few pieces spread over the order) and a pair of (T+8)^2 grid tiles in shared
+// memory, the one its current groups read and the one TMA fetches for the
+// next tile of its share (interior tiles; tiles that wrap around the grid
+// edge are loaded with plain loads when they are used).  The next group's
+// visibilities are loaded while the current one is computed.  Norms
+// accumulate per lane over a run and are summed once at its end.  No CTA
+// barrier separates the groups: with a CTA per work item (a tile's
+// visibilities of one block) and its barriers, warps waited at barriers for
+// 5 of every 14 cycles per issued instruction and small items left most
+// lanes idle.  Before -> now, with the dual step: 28.4 -> 16.8 us at 512^2
+// (524k visibilities), 159 -> 98 us at 1024^2 (4.2M), 42 -> 22 us at 640 x 480
+// (700k); without it 522 -> 237 us at 4096^2 (8.4M).  What bounds it now is
+// the shared-memory reads (64 eight-byte reads a visibility, two passes each
+// for a warp: 52 us of the SM's data path at 1024^2) and the issue slots
+// (61 % busy there).
 template <typename R> struct VisIn {
     VisRec<R> rc;
     cplx_t<R> v, y, p;
@@ -326,190 +327,152 @@ __device__ __forceinline__ void load_vis(const VisArgs<R> &A, int gi, VisIn<R> &
     }
 }
 
-// NTD threads per CTA (256 or 128; FP64: 256): the autotuner picks per
-// problem, fewer threads giving more CTAs per SM and shorter barriers.
-template <typename R, int T, int MODE, int NTD>
-__global__ void __launch_bounds__(NTD, sizeof(R) == 4 ? 768 / NTD : 1)
-    k_degrid(const __grid_constant__ CUtensorMap tmap, int use_tma, const cplx_t<R> *__restrict__ grid, VisArgs<R> A,
-             int n_units, long long spin_first) {
-    using C = cplx_t<R>;
-    constexpr int E = T + HALO;
-    constexpr int TILE_BYTES = E * E * (int)sizeof(C);
-    constexpr int TILE_STRIDE = (TILE_BYTES + 127) / 128 * 128;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t bar[2];
-    __shared__ int ok_s;
+// Warps per SM the degridding's shared memory and registers allow, and with
+// them the shares of the groups (a share per resident warp).  T = 32: one
+// tile buffer a warp (the copy is then waited for).
+template <typename R, int T> constexpr int dg_warps_per_sm() { return sizeof(R) == 8 ? 8 : T == 16 ? 24 : 16; }
+template <int T> constexpr int dg_bufs() { return T == 16 ? 2 : 1; }
 
-    if (threadIdx.x == 0) {
-        ok_s = 1;
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-    }
-    __syncthreads();
+// NTD threads per CTA (256 or 128; FP64: 256): the CTA only groups warps.
+template <typename R, int T, int MODE, int NTD>
+__global__ void __launch_bounds__(NTD, dg_warps_per_sm<R, T>() * 32 / NTD)
+    k_degrid(const __grid_constant__ CUtensorMap tmap, int use_tma, const cplx_t<R> *__restrict__ grid, VisArgs<R> A,
+             long long spin_first) {
+    using C = cplx_t<R>;
+    constexpr int E = T + HALO, NB = dg_bufs<T>();
+    constexpr int TILE_BYTES = E * E * (int)sizeof(C);
+    static_assert(TILE_BYTES % 128 == 0, "TMA destinations stay 128-byte aligned");
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ uint64_t bars[NTD / 32][NB];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned char *tiles = smem_raw + warp * NB * TILE_BYTES;
+    uint64_t *bar = bars[warp];
+    const int gw = blockIdx.x * (NTD / 32) + warp;   // this warp's share
+    if (lane == 0)
+        for (int k = 0; k < NB; ++k) mbar_init(&bar[k], 1);
+    __syncwarp();
     pdl_enter();   // the grid, v and p come from the kernels before
-    auto origin = [&](int u, int &row0, int &col0) {
-        const int tl = A.ch_tile[A.u_chunk[u]];
-        row0 = (tl / A.ntile1) * T;
-        col0 = (tl % A.ntile1) * T;
+    auto interior = [&](int tile) {
+        return use_tma && (tile / A.ntile1) * T + E <= A.K0 && (tile % A.ntile1) * T + E <= A.K1;
     };
-    auto interior = [&](int row0, int col0) { return use_tma && row0 + E <= A.K0 && col0 + E <= A.K1; };
-    auto issue = [&](int u, int buf) {   // thread 0 only
-        int r0, c0;
-        origin(u, r0, c0);
-        if (interior(r0, c0)) {
+    auto issue = [&](int tile, int buf) {   // lane 0 only
+        if (interior(tile)) {
             mbar_expect_tx(&bar[buf], (uint32_t)TILE_BYTES);
-            tma_load_2d(smem_raw + buf * TILE_STRIDE, &tmap, 2 * c0, r0, &bar[buf]);
+            tma_load_2d(tiles + buf * TILE_BYTES, &tmap, 2 * (tile % A.ntile1) * T, (tile / A.ntile1) * T, &bar[buf]);
         }
     };
-    uint32_t ph = 0u;   // bit b: parity of the next completion of bar[b]
-    const int32_t *ord = A.u_order;
-    __shared__ int claim_s, last_s, out_s;
-    auto claim = [&](int from) {   // thread 0: the next position after `from` (n_units: none)
-        claim_s = from < n_units ? (int)gridDim.x + atomicAdd(A.claim, 1) : n_units;
-    };
-    if (threadIdx.x == 0) {
-        if ((int)blockIdx.x < n_units) issue(ord[blockIdx.x], 0);
-        claim(blockIdx.x);
-    }
-    VisIn<R> cur;
-    if ((int)blockIdx.x < n_units && (int)threadIdx.x < A.u_count[ord[blockIdx.x]])
-        load_vis<R, MODE>(A, A.u_start[ord[blockIdx.x]] + threadIdx.x, cur);
-    __syncthreads();
-    int nxt_pos = min(claim_s, n_units);
-    int it = 0;
-    for (int iu = blockIdx.x; iu < n_units; iu = nxt_pos, nxt_pos = min(claim_s, n_units), ++it) {
-        const int buf = it & 1;
-        C *tile = reinterpret_cast<C *>(smem_raw + buf * TILE_STRIDE);
-        const int u = ord[iu];
-        const int nxt = nxt_pos < n_units ? ord[nxt_pos] : n_units;
-        if (threadIdx.x == 0 && nxt < n_units) issue(nxt, buf ^ 1);
-        const int start = A.u_start[u], count = A.u_count[u], ch = A.u_chunk[u];
-        int row0, col0;
-        origin(u, row0, col0);
-        if (interior(row0, col0)) {
-            // spin_first bounds the first wait (SPIN_LIMIT unless a test shortens
-            // it); the waits for copies in flight before leaving keep SPIN_LIMIT
-            if (!mbar_wait(&bar[buf], (ph >> buf) & 1u, spin_first)) {
-                atomicOr(A.err, ERR_TMA_TIMEOUT);
-                ok_s = 0;
-                mbar_wait(&bar[buf], (ph >> buf) & 1u, SPIN_LIMIT);   // second bounded wait for the copy in flight
-            }
-            ph ^= 1u << buf;
-            __syncthreads();
-            if (!ok_s) {
-                // the next unit's copy may be in flight: wait for it (bounded) before leaving
-                if (nxt < n_units) {
-                    int r1, c1;
-                    origin(nxt, r1, c1);
-                    if (interior(r1, c1)) mbar_wait(&bar[buf ^ 1], (ph >> (buf ^ 1)) & 1u, SPIN_LIMIT);
-                }
-                break;
-            }
-        } else {
-            for (int e = threadIdx.x; e < E * E; e += NTD) {
-                const int r = e / E, cc = e % E;
-                tile[e] = grid[(int64_t)((row0 + r) % A.K0) * A.K1 + (col0 + cc) % A.K1];
-            }
-            __syncthreads();
-        }
-        const int blk = A.ch_block[ch];
-        const R mu = (MODE != DG_OP) ? A.mu[blk] : R(0);
-        // block outside the active set D: z, w untouched (only the residual
-        // statistic is formed); block without a prox output yet: w = z, so
-        // that the next Algorithm 2 step starts from P_B(z)
-        const bool act = MODE == DG_OP || !A.bmask || A.bmask[blk];
-        const bool first_blk = MODE == DG_FIRST || (A.seen && !A.seen[blk]);
-        if (MODE != DG_OP && threadIdx.x == 0) {
-            if (A.inner_tol > 0) A.inner_state[blk] = 0;
-            if (A.inner_steps) A.inner_steps[blk] = act ? A.n_itr : 0;
-        }
-        // with the stopping test the start zbar^(0) = z of a block without a
-        // prox output is kept in p, the previous point of the first test
-        const bool keep_start = first_blk && A.inner_tol > 0;
+    const int g0 = gw < A.n_warps ? A.warp_grp[gw] : 0, g1 = gw < A.n_warps ? A.warp_grp[gw + 1] : 0;
+    if (g0 < g1) {
+        uint32_t ph = 0u;   // bit b: parity of the next completion of bar[b]
+        int4 D = A.grp[g0], Dn = D;   // {start, count, tile, block} of this group and the next
+        if (lane == 0) issue(D.z, 0);
+        VisIn<R> cur;
+        if (lane < D.y) load_vis<R, MODE>(A, D.x + lane, cur);
+        if (g0 + 1 < g1) Dn = A.grp[g0 + 1];
+        int buf = 0, run = A.warp_run[gw];
+        bool fresh = true;    // the group's tile has not been waited for
+        bool begin = true;    // the group starts a run
+        bool act = true, first_blk = MODE == DG_FIRST, keep_start = false;
+        R mu = 0;
         Acc<R> s_w, s_r;
-        for (int i = threadIdx.x; i < count; i += NTD) {
-            const int gi = start + i;
-            VisIn<R> nx;   // the next visibility: of this unit, else the next unit's first
-            if (i + NTD < count) load_vis<R, MODE>(A, gi + NTD, nx);
-            const int lb0 = (cur.rc.packed & 0xffff) - row0, lb1 = ((cur.rc.packed >> 16) & 0xffff) - col0;
-            R w0[KB_J], w1[KB_J];
-            kb_weights(cur.rc.f0, w0, A);
-            kb_weights(cur.rc.f1, w1, A);
-            C q{0, 0};
-#pragma unroll
-            for (int a = 0; a < KB_J; ++a) {
-                const C *row = tile + (lb0 + a) * E + lb1;
-                C r{0, 0};
-#pragma unroll
-                for (int b = 0; b < KB_J; ++b) {
-                    const C g = row[b];
-                    r.x += w1[b] * g.x;
-                    r.y += w1[b] * g.y;
+        for (int g = g0; g < g1; ++g) {
+            const bool more = g + 1 < g1, next_tile = more && Dn.z != D.z;
+            if (NB == 2 && next_tile && lane == 0) issue(Dn.z, buf ^ 1);
+            VisIn<R> nx;
+            if (more && lane < Dn.y) load_vis<R, MODE>(A, Dn.x + lane, nx);
+            const int4 Dn2 = g + 2 < g1 ? A.grp[g + 2] : Dn;
+            if (MODE != DG_OP && begin) {
+                const int blk = D.w;
+                mu = A.mu[blk];
+                // block outside the active set D: z, w untouched (only the
+                // residual statistic is formed); block without a prox output
+                // yet: w = z, so that the next Algorithm 2 step starts from P_B(z)
+                act = !A.bmask || A.bmask[blk];
+                first_blk = MODE == DG_FIRST || (A.seen && !A.seen[blk]);
+                // with the stopping test the start zbar^(0) = z of a block without
+                // a prox output is kept in p, the previous point of the first test
+                keep_start = first_blk && A.inner_tol > 0;
+                if (lane == 0) {
+                    if (A.inner_tol > 0) A.inner_state[blk] = 0;
+                    if (A.inner_steps) A.inner_steps[blk] = act ? A.n_itr : 0;
                 }
-                q.x += w0[a] * r.x;
-                q.y += w0[a] * r.y;
+                begin = false;
             }
-            const C phix{cur.th * q.x, cur.th * q.y};
-            if (MODE == DG_OP) {
-                A.op_out[A.perm ? A.perm[gi] : gi] = phix;
-            } else {
-                if (act) {
-                    const R invU = R(1) / cur.rc.U;
-                    const C zz{cur.v.x * invU + phix.x, cur.v.y * invU + phix.y};
-                    A.z[gi] = zz;
-                    C ww;
-                    if (first_blk) {
-                        ww = zz;
-                        if (keep_start) A.p[gi] = zz;
-                    } else {
-                        const R mu_u = mu * cur.rc.U;
-                        ww = C{cur.p.x - mu_u * (cur.p.x - zz.x), cur.p.y - mu_u * (cur.p.y - zz.y)};
+            C *tile = reinterpret_cast<C *>(tiles + buf * TILE_BYTES);
+            const int row0 = (D.z / A.ntile1) * T, col0 = (D.z % A.ntile1) * T;
+            if (fresh) {
+                if (interior(D.z)) {
+                    // spin_first bounds the first wait (SPIN_LIMIT unless a test shortens
+                    // it); the waits for copies in flight before leaving keep SPIN_LIMIT
+                    const bool ok = mbar_wait(&bar[buf], (ph >> buf) & 1u, spin_first);
+                    if (!__all_sync(0xffffffffu, ok)) {
+                        if (lane == 0) atomicOr(A.err, ERR_TMA_TIMEOUT);
+                        mbar_wait(&bar[buf], (ph >> buf) & 1u, SPIN_LIMIT);
+                        if (NB == 2 && next_tile && interior(Dn.z))
+                            mbar_wait(&bar[buf ^ 1], (ph >> (buf ^ 1)) & 1u, SPIN_LIMIT);
+                        break;
                     }
-                    A.w[gi] = ww;
-                    const R dx = ww.x - cur.y.x, dy = ww.y - cur.y.y;
-                    s_w.add(dx * dx + dy * dy);
+                    ph ^= 1u << buf;
+                } else {
+                    for (int e = lane; e < E * E; e += 32) {
+                        const int r = e / E, cc = e % E;
+                        tile[e] = grid[(int64_t)((row0 + r) % A.K0) * A.K1 + (col0 + cc) % A.K1];
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // a later copy refills the buffer
+                    __syncwarp();
                 }
-                const R ex = phix.x - cur.y.x, ey = phix.y - cur.y.y;
-                s_r.add(ex * ex + ey * ey);
+                fresh = false;
             }
-            if (i + NTD < count) cur = nx;
-        }
-        // this thread's first visibility of the next unit (loaded during the
-        // unit's reduction and barrier below)
-        if (nxt < n_units && (int)threadIdx.x < A.u_count[nxt]) load_vis<R, MODE>(A, A.u_start[nxt] + threadIdx.x, cur);
-        // the position after the next unit (read after the barrier below;
-        // rewritten only after the next unit's first barrier)
-        if (threadIdx.x == 0) claim(nxt_pos);
-        if constexpr (MODE != DG_OP) {
-            const decltype(s_w.get()) part[2] = {s_w.get(), s_r.get()};
-            double sum[2];
-            cta_sums<NTD>(part, sum);
-            if (threadIdx.x == 0) {
-                double *out = A.partials + NPART * (int64_t)A.u_pos[u];
-                out[0] = sum[0];
-                out[1] = sum[1];
-                last_s = unit_done(A, blk);
+            if (lane < D.y) {
+                const int gi = D.x + lane;
+                const int lb0 = (cur.rc.packed & 0xffff) - row0, lb1 = ((cur.rc.packed >> 16) & 0xffff) - col0;
+                R w0[KB_J], w1[KB_J];
+                kb_weights(cur.rc.f0, w0, A);
+                kb_weights(cur.rc.f1, w1, A);
+                const C q = footprint<E>(tile + lb0 * E + lb1, w0, w1);
+                const C phix{cur.th * q.x, cur.th * q.y};
+                if (MODE == DG_OP) {
+                    A.op_out[A.perm ? A.perm[gi] : gi] = phix;
+                } else {
+                    if (act) {
+                        const R invU = R(1) / cur.rc.U;
+                        const C zz{cur.v.x * invU + phix.x, cur.v.y * invU + phix.y};
+                        A.z[gi] = zz;
+                        C ww;
+                        if (first_blk) {
+                            ww = zz;
+                            if (keep_start) A.p[gi] = zz;
+                        } else {
+                            const R mu_u = mu * cur.rc.U;
+                            ww = C{cur.p.x - mu_u * (cur.p.x - zz.x), cur.p.y - mu_u * (cur.p.y - zz.y)};
+                        }
+                        A.w[gi] = ww;
+                        const R dx = ww.x - cur.y.x, dy = ww.y - cur.y.y;
+                        s_w.add(dx * dx + dy * dy);
+                    }
+                    const R ex = phix.x - cur.y.x, ey = phix.y - cur.y.y;
+                    s_r.add(ex * ex + ey * ey);
+                }
             }
+            if (MODE != DG_OP && (!more || Dn.w != D.w)) {   // the run ends
+                const decltype(s_w.get()) part[2] = {s_w.get(), s_r.get()};
+                const auto t = warp_sums<2>(part);
+                if (lane % 16 == 0) A.partials[NPART * (int64_t)A.run_pos[run] + lane / 16] = as_double(t);
+                ++run;
+                s_w = Acc<R>{};
+                s_r = Acc<R>{};
+                begin = true;
+            }
+            if (next_tile) {
+                __syncwarp();   // every lane has read the tile: its buffer may be refilled
+                if (NB == 2) buf ^= 1;
+                else if (lane == 0) issue(Dn.z, 0);
+                fresh = true;
+            }
+            D = Dn;
+            Dn = Dn2;
+            cur = nx;
         }
-        __syncthreads();   // the tile buffer is refilled two units later
-        if constexpr (MODE != DG_OP) {
-            if (last_s) block_scale<NTD>(A, blk, false);
-        }
-    }
-    // no claim follows this CTA's exit: the last CTA out resets the counters
-    // (the blocks' too: a launch whose wait ran out leaves units undone)
-    if (threadIdx.x == 0) {
-        __threadfence();
-        out_s = atomicAdd(A.claim + 1, 1) == (int)gridDim.x - 1;
-        if (out_s) {
-            A.claim[0] = 0;
-            A.claim[1] = 0;
-        }
-    }
-    if constexpr (MODE != DG_OP) {
-        __syncthreads();
-        if (out_s)
-            for (int j = threadIdx.x; j < A.n_blocks; j += NTD) A.blk_done[j] = 0;
     }
 }
 
@@ -525,63 +488,154 @@ __global__ void __launch_bounds__(NTD, sizeof(R) == 4 ? 768 / NTD : 1)
 // Stopping test (inner_tol > 0): p is kept every step; a step k >= 1 also
 // forms the partials ||p - p_prev||^2 and ||p||^2; a block whose test held
 // for the previous step (or earlier) stops, its p being the prox output.
+// The work is split as in the degridding (a warp per share of the groups).
+constexpr int SUB_NT = 256;
 template <typename R>
-__global__ void __launch_bounds__(DG_NT) k_subiter(VisArgs<R> A, int only_first, R beta, int write_p) {
+__global__ void __launch_bounds__(SUB_NT) k_subiter(VisArgs<R> A, int only_first, R beta, int write_p) {
     using C = cplx_t<R>;
-    const int u = blockIdx.x;   // one work unit (at most DG_NT visibilities)
-    const int start = A.u_start[u], count = A.u_count[u], blk = A.ch_block[A.u_chunk[u]];
+    const int lane = threadIdx.x & 31, gw = blockIdx.x * (SUB_NT / 32) + (threadIdx.x >> 5);
     pdl_enter();
-    const bool act = !A.bmask || A.bmask[blk];
-    const bool first_blk = A.seen && !A.seen[blk];
-    if (!act || (only_first && !first_blk)) return;   // (the same for every unit of the block)
     const bool tol_on = A.inner_tol > 0;
-    // stopped at an earlier step of this iteration (this launch's own mark
-    // comes after every unit of the block has finished)
-    if (tol_on && A.inner_state[blk]) return;
-    const R c = A.scale[blk];
-    const R mu = A.mu[blk];
+    // blocks this step leaves as they are: outside D, not first in an
+    // only_first step, or stopped at an earlier step of this iteration
+    auto skips = [&](int blk) {
+        return (A.bmask && !A.bmask[blk]) || (only_first && !(A.seen && !A.seen[blk])) ||
+               (tol_on && A.inner_state[blk]);
+    };
     const bool test_out = tol_on && A.step > 0;
-    const bool keep = write_p || tol_on;
-    Acc<R> s_w, s_d, s_n;
-    for (int i = threadIdx.x; i < count; i += DG_NT) {
-        const int gi = start + i;
-        const R U = A.rec[gi].U;
-        const C yy = A.y[gi], ww = A.w[gi], zz = A.z[gi];
-        const C pp{yy.x + c * (ww.x - yy.x), yy.y + c * (ww.y - yy.y)};
-        C q = pp;
-        if (beta != R(0) || test_out) {
-            const C pm = A.p[gi];
-            if (beta != R(0)) q = C{pp.x + beta * (pp.x - pm.x), pp.y + beta * (pp.y - pm.y)};
-            if (test_out) {
-                const R ex = pp.x - pm.x, ey = pp.y - pm.y;
-                s_d.add(ex * ex + ey * ey);
-                s_n.add(pp.x * pp.x + pp.y * pp.y);
+    const bool keep = write_p || tol_on, prev = beta != R(0) || test_out;
+    const int g0 = gw < A.n_warps ? A.warp_grp[gw] : 0, g1 = gw < A.n_warps ? A.warp_grp[gw + 1] : 0;
+    struct In {
+        R U;
+        C y, w, z, p;
+    };
+    auto load = [&](int gi, In &o) {
+        o.U = A.rec[gi].U;
+        o.y = A.y[gi];
+        o.w = A.w[gi];
+        o.z = A.z[gi];
+        if (prev) o.p = A.p[gi];
+    };
+    if (g0 < g1) {
+        int run = A.warp_run[gw];
+        int4 D = A.grp[g0];
+        In cur;
+        if (lane < D.y) load(D.x + lane, cur);
+        bool begin = true, skip = false;
+        R c = 0, mu = 0;
+        Acc<R> s_w, s_d, s_n;
+        for (int g = g0; g < g1; ++g) {
+            const bool more = g + 1 < g1;
+            const int4 Dn = more ? A.grp[g + 1] : D;
+            In nx;
+            if (more && lane < Dn.y) load(Dn.x + lane, nx);
+            if (begin) {
+                skip = skips(D.w);
+                c = A.scale[D.w];
+                mu = A.mu[D.w];
+                begin = false;
             }
+            if (!skip && lane < D.y) {
+                const int gi = D.x + lane;
+                const C yy = cur.y, ww = cur.w, zz = cur.z;
+                const C pp{yy.x + c * (ww.x - yy.x), yy.y + c * (ww.y - yy.y)};
+                C q = pp;
+                if (prev) {
+                    const C pm = cur.p;
+                    if (beta != R(0)) q = C{pp.x + beta * (pp.x - pm.x), pp.y + beta * (pp.y - pm.y)};
+                    if (test_out) {
+                        const R ex = pp.x - pm.x, ey = pp.y - pm.y;
+                        s_d.add(ex * ex + ey * ey);
+                        s_n.add(pp.x * pp.x + pp.y * pp.y);
+                    }
+                }
+                if (keep) A.p[gi] = pp;
+                const R mu_u = mu * cur.U;
+                const C wn{q.x - mu_u * (q.x - zz.x), q.y - mu_u * (q.y - zz.y)};
+                A.w[gi] = wn;
+                const R dx = wn.x - yy.x, dy = wn.y - yy.y;
+                s_w.add(dx * dx + dy * dy);
+            }
+            if (!more || Dn.w != D.w) {   // the run ends
+                if (!skip) {
+                    const decltype(s_w.get()) part[3] = {s_w.get(), s_d.get(), s_n.get()};
+                    const auto t = warp_sums<3>(part);
+                    // slot 1 keeps the degridding's residual
+                    if (lane % 8 == 0 && lane < 24)
+                        A.partials[NPART * (int64_t)A.run_pos[run] + (lane ? lane / 8 + 1 : 0)] = as_double(t);
+                }
+                ++run;
+                s_w = s_d = s_n = Acc<R>{};
+                begin = true;
+            }
+            D = Dn;
+            cur = nx;
         }
-        if (keep) A.p[gi] = pp;
-        const R mu_u = mu * U;
-        const C wn{q.x - mu_u * (q.x - zz.x), q.y - mu_u * (q.y - zz.y)};
-        A.w[gi] = wn;
-        const R dx = wn.x - yy.x, dy = wn.y - yy.y;
-        s_w.add(dx * dx + dy * dy);
     }
-    __shared__ int last_s;
-    const decltype(s_w.get()) part[3] = {s_w.get(), s_d.get(), s_n.get()};
-    double sum[3];
-    cta_sums<DG_NT>(part, sum);
-    if (threadIdx.x == 0) {
-        double *out = A.partials + NPART * (int64_t)A.u_pos[u];
-        out[0] = sum[0];
-        out[2] = sum[1];
-        out[3] = sum[2];
-        last_s = unit_done(A, blk);
-        if (last_s) A.blk_done[blk] = 0;
-    }
-    __syncthreads();
-    if (last_s) block_scale<DG_NT>(A, blk, test_out);
 }
 
 // ----------------------------------------------------------------- block norms
+// P_B scale of every block after the degridding or a sub-iteration (Section
+// 3.3, Eq. "proj-L2" as a radial scale): eps / ||w - y|| if that norm exceeds
+// eps, else 1, from the block's norm partials summed in FP64 in a fixed
+// order, a CTA per block.  After a sub-iteration with the stopping test
+// (step > 0): ||zbar^t - zbar^(t-1)|| <= inner_tol ||zbar^t|| in FP64; a block
+// whose test holds is marked stopped at this step (a block that stopped
+// before, or that the step left alone, keeps what it has: its partials are
+// those of its last step).
+// A launch of its own: in the prologue of every CTA of the next kernel the
+// sums took 19 of the gridding's 46 us at 512^2 with 16 blocks and 45 of a
+// sub-iteration's 61 us (640 x 480, 12 blocks), their FP64 adds queueing for
+// the SM's two FP64 lanes; in the CTA that counted a block's last run, the
+// last CTA found most blocks at once (7 us after the others at 512^2, 35 us
+// at 1024^2 with 64 blocks).
+constexpr int BS_NT = 256;
+template <typename R>
+__global__ void __launch_bounds__(BS_NT) k_block_scale(const double *__restrict__ partials,
+                                                       const int32_t *__restrict__ blk_ptr,
+                                                       const double *__restrict__ eps, double inner_tol, int step,
+                                                       R *__restrict__ scale, int *__restrict__ inner_state,
+                                                       int *__restrict__ err) {
+    __shared__ double red[BS_NT / 32][3];
+    const int blk = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_enter();
+    const int k0 = blk_ptr[blk], k1 = blk_ptr[blk + 1];
+    const bool test = inner_tol > 0 && step > 0;
+    double v[3] = {0, 0, 0};
+#pragma unroll 8
+    for (int k = k0 + threadIdx.x; k < k1; k += BS_NT) v[0] += partials[NPART * (int64_t)k];
+    if (test)
+#pragma unroll 4
+        for (int k = k0 + threadIdx.x; k < k1; k += BS_NT) {
+            v[1] += partials[NPART * (int64_t)k + 2];
+            v[2] += partials[NPART * (int64_t)k + 3];
+        }
+    const int nw = min(BS_NT / 32, (k1 - k0 + 31) / 32);   // warps with a partial
+    if (warp < nw) {
+        if (test) {
+            const double t = warp_sums<3>(v);
+            if (lane % 8 == 0 && lane < 24) red[warp][lane / 8] = t;
+        } else {
+            const double u[1] = {v[0]}, t = warp_sums<1>(u);
+            if (lane == 0) red[warp][0] = t;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double a = 0, d = 0, n = 0;
+        for (int w = 0; w < nw; ++w) a += red[w][0];
+        if (test)
+            for (int w = 0; w < nw; ++w) {
+                d += red[w][1];
+                n += red[w][2];
+            }
+        const double nrm = sqrt(a);
+        if (!isfinite(nrm)) atomicOr(err, ERR_NONFINITE);
+        scale[blk] = (R)((nrm > eps[blk]) ? eps[blk] / nrm : 1.0);
+        if (test && inner_state[blk] == 0 && sqrt(d) <= inner_tol * sqrt(n)) inner_state[blk] = step;
+    }
+}
+
 // One warp per block j: ||Phi_j xt - y_j||^2 of the last data step from the
 // block's partials (fixed order), for the statistics and the stopping rule.
 __global__ void k_block_norms(const double *__restrict__ partials, const int32_t *__restrict__ blk_ptr, int d,
@@ -896,17 +950,14 @@ template <typename R> VisArgs<R> make_args(ppd_ctx *c) {
     A.w = static_cast<cplx_t<R> *>(c->w);
     A.p = static_cast<cplx_t<R> *>(c->p);
     A.mu = static_cast<const R *>(c->mu_d);
-    A.scale = static_cast<R *>(c->scale);
-    A.blk_done = c->blk_done;
-    A.n_blocks = c->d;
+    A.scale = static_cast<const R *>(c->scale);
     A.partials = c->partials;
     A.blk_ptr = c->ch.blk_ptr;
-    A.u_pos = c->ch.u_pos;
-    A.u_start = c->ch.u_start;
-    A.u_count = c->ch.u_count;
-    A.u_chunk = c->ch.u_chunk;
-    A.u_order = c->ch.u_order;
-    A.claim = c->dg_claim;
+    A.run_pos = c->ch.run_pos;
+    A.warp_run = c->ch.warp_run;
+    A.grp = c->ch.grp;
+    A.warp_grp = c->ch.warp_grp;
+    A.n_warps = c->ch.n_warps;
     A.eps = c->eps_d;
     A.err = c->err;
     A.bmask = c->rand_on ? c->mask_cur : nullptr;
@@ -926,34 +977,38 @@ template <typename R, int T, int NW> size_t grid_smem() {
            (size_t)NW * KB_J * SP * sizeof(R);
 }
 
+// the blocks' scales from the norm partials of the kernel before
+template <typename R> int block_scales(ppd_ctx *c, int step, cudaStream_t s) {
+    int site;
+    PPD_CHECK(launch_begin(c, "block_scale", s, &site));
+    launch(c, true, k_block_scale<R>, (unsigned)c->d, BS_NT, 0, s, (const double *)c->partials,
+           (const int32_t *)c->ch.blk_ptr, (const double *)c->eps_d, c->cfg.inner_tol, step,
+           static_cast<R *>(c->scale), c->inner_state, c->err);
+    return launch_end(c, site, s);
+}
+
 template <typename R, int T, int NTD>
 int degrid_t(ppd_ctx *c, int mode, const cplx_t<R> *grid, cplx_t<R> *out, const int64_t *perm, cudaStream_t s) {
     VisArgs<R> A = make_args<R>(c);
     A.op_out = out;
     A.perm = perm;
     constexpr int E = T + HALO;
-    const size_t tile_stride = ((size_t)E * E * sizeof(cplx_t<R>) + 127) / 128 * 128;
-    const size_t sh = 2 * tile_stride;
+    const size_t sh = (size_t)(NTD / 32) * dg_bufs<T>() * E * E * sizeof(cplx_t<R>);
     PPD_CHECK(smem_attr((const void *)k_degrid<R, T, DG_OP, NTD>, (int)sh));
     PPD_CHECK(smem_attr((const void *)k_degrid<R, T, DG_DUAL, NTD>, (int)sh));
     PPD_CHECK(smem_attr((const void *)k_degrid<R, T, DG_FIRST, NTD>, (int)sh));
     const int use_tma = (c->tma_ok && grid == c->grid_a) ? 1 : 0;
-    if (c->ch.nu == 0) return PPD_OK;
-    int per_sm = 0;
-    PPD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_degrid<R, T, DG_DUAL, NTD>, NTD, sh));
-    if (per_sm < 1) per_sm = 1;
-    int sms = 0;
-    PPD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
-    const int nch = (int)c->ch.nu;   // work units
-    const unsigned nb = (unsigned)std::min<int64_t>(nch, (int64_t)sms * per_sm);
+    if (c->ch.n_grp == 0) return PPD_OK;
+    const unsigned nb = (unsigned)((c->ch.n_warps + NTD / 32 - 1) / (NTD / 32));
     int site;
     PPD_CHECK(launch_begin(c, mode == DG_OP ? "degrid_op" : "degrid_dual", s, &site));
     const long long sf = c->wait_first;
     auto k = mode == DG_OP     ? k_degrid<R, T, DG_OP, NTD>
              : mode == DG_DUAL ? k_degrid<R, T, DG_DUAL, NTD>
                                : k_degrid<R, T, DG_FIRST, NTD>;
-    launch(c, true, k, nb, NTD, sh, s, c->tmap_a, use_tma, grid, A, nch, sf);
-    return launch_end(c, site, s);
+    launch(c, true, k, nb, NTD, sh, s, c->tmap_a, use_tma, grid, A, sf);
+    PPD_CHECK(launch_end(c, site, s));
+    return mode == DG_OP ? PPD_OK : block_scales<R>(c, 0, s);
 }
 
 template <typename R, int T, int NW> int grid_launch(ppd_ctx *c, int mode, const VisArgs<R> &A, cudaStream_t s) {
@@ -994,6 +1049,11 @@ int grid_t(ppd_ctx *c, int mode, const cplx_t<R> *in, const int64_t *perm, cplx_
 }
 
 }  // namespace
+
+int degrid_warps_per_sm(const ppd_ctx *c) {
+    if (!c->is_f32) return c->T == 16 ? dg_warps_per_sm<double, 16>() : dg_warps_per_sm<double, 32>();
+    return c->T == 16 ? dg_warps_per_sm<float, 16>() : dg_warps_per_sm<float, 32>();
+}
 
 // Binning entry used by the API: fills key, base (2 per vis), frac (2 per
 // vis), per-visibility cell count.
@@ -1114,11 +1174,13 @@ int grid_vis(ppd_ctx *c, int mode, const cplx_t<R> *in, const int64_t *perm, cpl
 }
 
 template <typename R> int subiter(ppd_ctx *c, cudaStream_t s, int only_first, double beta, int write_p) {
-    if (c->ch.nu == 0) return PPD_OK;
+    if (c->ch.n_grp == 0) return PPD_OK;
     int site;
     PPD_CHECK(launch_begin(c, "subiter", s, &site));
-    launch(c, true, k_subiter<R>, (unsigned)c->ch.nu, DG_NT, 0, s, make_args<R>(c), only_first, (R)beta, write_p);
-    return launch_end(c, site, s);
+    const unsigned nb = (unsigned)((c->ch.n_warps + SUB_NT / 32 - 1) / (SUB_NT / 32));
+    launch(c, true, k_subiter<R>, nb, SUB_NT, 0, s, make_args<R>(c), only_first, (R)beta, write_p);
+    PPD_CHECK(launch_end(c, site, s));
+    return block_scales<R>(c, c->next_step, s);
 }
 
 int block_norms(ppd_ctx *c, cudaStream_t s) {
