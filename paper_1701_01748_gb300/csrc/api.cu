@@ -122,8 +122,7 @@ void dfree(void *p) {
 
 void free_vis(ppd_ctx *c) {
     for (void *p : {c->rec, c->theta_v, c->y, c->v, c->z, c->w, c->p, c->y_raw, (void *)c->perm,
-                    (void *)c->count_cell, (void *)c->ch.start, (void *)c->ch.count, (void *)c->ch.tile,
-                    (void *)c->ch.block, (void *)c->ch.tile_first, (void *)c->ch.tile_n, (void *)c->ch.blk_ptr,
+                    (void *)c->count_cell, (void *)c->ch.gg, (void *)c->ch.it_grp, (void *)c->ch.tile_first, (void *)c->ch.tile_n, (void *)c->ch.blk_ptr,
                     (void *)c->ch.grp, (void *)c->ch.warp_grp, (void *)c->ch.warp_run, (void *)c->ch.run_pos, (void *)c->ch.order, (void *)c->ch.active, (void *)c->partials, c->scale, (void *)c->resid2,
                     (void *)c->eps_d, c->mu_d, c->gpart})
         dfree(p);
@@ -877,28 +876,35 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     }
     const uint64_t KK = (uint64_t)c->K0 * c->K1;
     const int ntiles = (c->K0 / c->T) * (c->K1 / c->T);
-    std::vector<int32_t> cs, cn, ct, cbk, tfirst(ntiles, 0), tn(ntiles, 0);
-    std::vector<int4> grp;   // groups of the degridding and sub-iterations
+    // groups of at most 32 visibilities of one tile and block, and gridding
+    // work items: groups of one tile up to C visibilities
+    std::vector<int32_t> tfirst(ntiles, 0), tn(ntiles, 0), in;
+    std::vector<int4> grp;
+    std::vector<int2> it;
+    const int gsz = std::min(32, c->C);
+    int64_t n_tb = 0;
     for (int64_t i = 0; i < M;) {
         const uint64_t k0 = key[c->perm_h[i]];
         const uint64_t tb = k0 / KK;   // tile * d + block
         int64_t j = i;
         while (j < M && key[c->perm_h[j]] / KK == tb) ++j;
-        for (int64_t s = i; s < j; s += c->C) {
-            const int tile = (int)(tb / (uint64_t)c->d), blk = (int)(tb % (uint64_t)c->d);
-            if (tn[tile] == 0) tfirst[tile] = (int32_t)cs.size();
-            tn[tile]++;
-            cs.push_back((int32_t)s);
-            cn.push_back((int32_t)std::min<int64_t>(c->C, j - s));
-            ct.push_back(tile);
-            cbk.push_back(blk);
+        const int tile = (int)(tb / (uint64_t)c->d), blk = (int)(tb % (uint64_t)c->d);
+        n_tb += (j - i + c->C - 1) / c->C;
+        for (int64_t s = i; s < j; s += gsz) {
+            const int n = (int)std::min<int64_t>(gsz, j - s);
+            if (tn[tile] == 0 || in.back() + n > c->C) {
+                if (tn[tile]++ == 0) tfirst[tile] = (int32_t)it.size();
+                it.push_back(make_int2((int)grp.size(), 0));
+                in.push_back(0);
+            }
+            it.back().y++;
+            in.back() += n;
+            grp.push_back(make_int4((int)s, n, tile, blk));
         }
-        for (int64_t s = i; s < j; s += 32)
-            grp.push_back(make_int4((int)s, (int)std::min<int64_t>(32, j - s), (int)(tb / (uint64_t)c->d),
-                                    (int)(tb % (uint64_t)c->d)));
         i = j;
     }
-    const int64_t nch = (int64_t)cs.size();
+    const int64_t nch = (int64_t)it.size();
+    const std::vector<int4> gg = grp;   // (the degridding's copy is reordered below)
     // tiles the gridding can reach: a tile with chunks and the tiles below,
     // right and below-right of it (the extended footprint's halo)
     std::vector<int32_t> active;
@@ -975,11 +981,18 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
         std::vector<int32_t> fill(bptr.begin(), bptr.end() - 1);
         for (int64_t r = 0; r < nruns; ++r) rpos[r] = fill[rblk[r]]++;
     }
-    // the gridding's CTA order: chunks by decreasing size
+    // the gridding's order: items by decreasing number of groups.  Items of
+    // up to `small` groups take one warp; with too few groups to fill the
+    // GPU's warps several times over, larger ones already spread over a CTA
     std::vector<int32_t> cord(nch);
     for (int64_t k = 0; k < nch; ++k) cord[k] = (int32_t)k;
-    std::stable_sort(cord.begin(), cord.end(), [&](int32_t a, int32_t b) { return cn[a] > cn[b]; });
+    std::stable_sort(cord.begin(), cord.end(), [&](int32_t a, int32_t b) { return it[a].y > it[b].y; });
+    const int small = ng >= 64LL * std::max(sms, 1) ? 4 : 1;
+    int64_t n_large = 0;
+    while (n_large < nch && it[cord[n_large]].y > small) ++n_large;
     c->ch.n = nch;
+    c->ch.n_large = n_large;
+    c->ch.n_tb = n_tb;
     c->ch.n_grp = (int32_t)ng;
     c->ch.n_warps = (int32_t)nwarps;
     c->ch.n_runs = nruns;
@@ -992,8 +1005,8 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     c->ch.n_active = (int64_t)active.size();
     const size_t cbsz = 2 * c->rsz;
     const int E = c->T + HALO;
-    if ((st = dalloc(&c->ch.start, nch)) || (st = dalloc(&c->ch.count, nch)) || (st = dalloc(&c->ch.tile, nch)) ||
-        (st = dalloc(&c->ch.block, nch)) || (st = dalloc(&c->ch.tile_first, ntiles)) ||
+    if ((st = dalloc(&c->ch.gg, ng)) || (st = dalloc(&c->ch.it_grp, nch)) ||
+        (st = dalloc(&c->ch.tile_first, ntiles)) ||
         (st = dalloc(&c->ch.tile_n, ntiles)) || (st = dalloc(&c->ch.blk_ptr, c->d + 1)) ||
         (st = dalloc(&c->ch.grp, ng)) || (st = dalloc(&c->ch.warp_grp, nwarps + 1)) || (st = dalloc(&c->ch.warp_run, nwarps + 1)) ||
         (st = dalloc(&c->ch.run_pos, nruns)) ||
@@ -1025,10 +1038,8 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
         const int cb0 = (base[2 * o] + c->K0 / 2) % c->K0, cb1 = (base[2 * o + 1] + c->K1 / 2) % c->K1;
         c->packed_h[i] = cb0 | (cb1 << 16);
     }
-    if ((e = cudaMemcpy(c->ch.start, cs.data(), nch * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->ch.count, cn.data(), nch * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->ch.tile, ct.data(), nch * 4, cudaMemcpyHostToDevice)) ||
-        (e = cudaMemcpy(c->ch.block, cbk.data(), nch * 4, cudaMemcpyHostToDevice)) ||
+    if ((e = cudaMemcpy(c->ch.gg, gg.data(), ng * sizeof(int4), cudaMemcpyHostToDevice)) ||
+        (e = cudaMemcpy(c->ch.it_grp, it.data(), nch * sizeof(int2), cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(c->ch.tile_first, tfirst.data(), ntiles * 4, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(c->ch.tile_n, tn.data(), ntiles * 4, cudaMemcpyHostToDevice)) ||
         (e = cudaMemcpy(c->ch.blk_ptr, bptr.data(), (c->d + 1) * 4, cudaMemcpyHostToDevice)) ||
@@ -1292,7 +1303,7 @@ int ppd_get_params(ppd_ctx *c, ppd_params *o) {
     o->chunk = c->C;
     o->grid_warps = c->grid_nw;
     o->degrid_threads = c->degrid_nt;
-    o->n_chunks = c->ch.n;
+    o->n_chunks = c->ch.n_tb;
     o->M = c->M;
     o->psiw_norm_sq = c->psiw2;
     o->alpha = c->kappa * c->psiw2;

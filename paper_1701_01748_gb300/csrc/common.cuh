@@ -15,8 +15,9 @@
 //                record {packed centred base cell, frac0, frac1, U} and the
 //                complex arrays y (whitened), v (dual), z, w (Algorithm 2
 //                work) and p (prox output, warm start)
-//   work items   "chunks": runs of <= chunk visibilities sharing one tile and
-//                one block; every gridding/degridding CTA owns one chunk
+//   work         groups of <= 32 visibilities sharing one tile and one block,
+//                shared out to the degridding warps; gridding work items:
+//                sequences of groups of one tile (<= chunk visibilities)
 #pragma once
 
 #include <cuda.h>
@@ -136,8 +137,16 @@ FftPlan make_fft_plan(int K);
 bool fft_length_supported(int K, bool fp64);
 
 struct Chunks {
-    int64_t n = 0;
-    int32_t *start = nullptr, *count = nullptr, *tile = nullptr, *block = nullptr;   // device
+    // gridding work items: sequences of groups of one tile with at most C
+    // visibilities, in the processing order (item k: it_grp[k].y groups of gg
+    // from it_grp[k].x on; tile t: items tile_first[t] .. + tile_n[t] - 1);
+    // order lists them by decreasing size, the first n_large get a CTA each,
+    // the others a warp each.  n_tb: runs of at most C visibilities of one
+    // tile and block (ppd_params.n_chunks; the fixed scratch of
+    // ppd_op_adjoint_noalloc is checked against that many partial tiles).
+    int64_t n = 0, n_large = 0, n_tb = 0;
+    int4 *gg = nullptr;
+    int2 *it_grp = nullptr;
     int32_t *tile_first = nullptr, *tile_n = nullptr;                                // device, n_tiles
     // work of the degridding and sub-iterations: groups of at most 32
     // visibilities of one tile and block {start, count, tile, block}, shared
@@ -150,7 +159,7 @@ struct Chunks {
     int4 *grp = nullptr;
     int32_t *warp_grp = nullptr, *warp_run = nullptr, *run_pos = nullptr;
     int32_t *blk_ptr = nullptr;
-    int32_t *order = nullptr;    // chunks by decreasing size (the gridding's CTA order)
+    int32_t *order = nullptr;
     int32_t *active = nullptr;   // tiles the combine pass writes (device)
     int64_t n_active = 0;
 };

@@ -58,7 +58,7 @@ extern "C" int ppd_op_adjoint_noalloc(ppd_ctx *c, const void *y_dev, void *x_dev
     if (!c || !y_dev || !x_dev) return fail(PPD_ERR_INVALID_ARG, "ppd_op_adjoint_noalloc: NULL argument");
     if (!c->have_weights) return fail(PPD_ERR_NOT_READY, "ppd_op_adjoint_noalloc: call ppd_set_weights first");
     const size_t E = (size_t)(c->T + HALO);
-    const size_t need = (size_t)c->ch.n * E * E * 2 * c->rsz;
+    const size_t need = (size_t)c->ch.n_tb * E * E * 2 * c->rsz;
     if (need > (size_t)PPD_NOALLOC_SCRATCH_BYTES)
         return fail(PPD_ERR_UNSUPPORTED,
                     "ppd_op_adjoint_noalloc: problem needs " + std::to_string(need) +

@@ -121,8 +121,12 @@ template <typename R> struct VisArgs {
     const VisRec<R> *rec;
     const R *theta_v;
     R theta_s;
-    const int32_t *ch_start, *ch_count, *ch_tile, *ch_block;
-    const int32_t *ch_order;   // chunks by decreasing size: the gridding's CTA order
+    // gridding work items (sequences of groups of one tile): item k owns the
+    // it_grp[k].y groups of gg (groups in the processing order) from
+    // it_grp[k].x on; it_order: the items by decreasing size
+    const int4 *gg;
+    const int2 *it_grp;
+    const int32_t *it_order;
     // groups of at most 32 visibilities of one tile and block {start, count,
     // tile, block}: warp w of the degridding and sub-iteration kernels owns
     // groups warp_grp[w] .. warp_grp[w + 1] - 1; its maximal sequences of
@@ -158,8 +162,7 @@ template <typename R> struct VisArgs {
     // (0: the step that forms the start P_B(z); 1 .. n_itr - 1: sub-iterations;
     // n_itr: the gridding), per block the step at which the test held (0:
     // running) and the steps taken
-    double inner_tol;
-    int step, n_itr;
+    int tol_on, step, n_itr;
     int *inner_state, *inner_steps;
 };
 
@@ -237,7 +240,7 @@ template <int NV, typename V> __device__ __forceinline__ V warp_sums(const V (&i
 // a w + c on both components: one instruction on packed pairs in FP32 (the
 // same two roundings as two fmaf), half the issue slots of the taps' sums
 struct F32x2 {
-    unsigned long long v;
+    unsigned long long v = 0;
 };
 __device__ __forceinline__ F32x2 pack2(float x, float y) {
     F32x2 r;
@@ -391,9 +394,9 @@ __global__ void __launch_bounds__(NTD, dg_warps_per_sm<R, T>() * 32 / NTD)
                 first_blk = MODE == DG_FIRST || (A.seen && !A.seen[blk]);
                 // with the stopping test the start zbar^(0) = z of a block without
                 // a prox output is kept in p, the previous point of the first test
-                keep_start = first_blk && A.inner_tol > 0;
+                keep_start = first_blk && A.tol_on;
                 if (lane == 0) {
-                    if (A.inner_tol > 0) A.inner_state[blk] = 0;
+                    if (A.tol_on) A.inner_state[blk] = 0;
                     if (A.inner_steps) A.inner_steps[blk] = act ? A.n_itr : 0;
                 }
                 begin = false;
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__(SUB_NT) k_subiter(VisArgs<R> A, int only_first
     using C = cplx_t<R>;
     const int lane = threadIdx.x & 31, gw = blockIdx.x * (SUB_NT / 32) + (threadIdx.x >> 5);
     pdl_enter();
-    const bool tol_on = A.inner_tol > 0;
+    const bool tol_on = A.tol_on;
     // blocks this step leaves as they are: outside D, not first in an
     // only_first step, or stopped at an earlier step of this iteration
     auto skips = [&](int blk) {
@@ -580,7 +583,7 @@ __global__ void __launch_bounds__(SUB_NT) k_subiter(VisArgs<R> A, int only_first
 // eps, else 1, from the block's norm partials summed in FP64 in a fixed
 // order, a CTA per block.  After a sub-iteration with the stopping test
 // (step > 0): ||zbar^t - zbar^(t-1)|| <= inner_tol ||zbar^t|| in FP64; a block
-// whose test holds is marked stopped at this step (a block that stopped
+// whose test holds is marked stopped at this step, its last (a block that stopped
 // before, or that the step left alone, keeps what it has: its partials are
 // those of its last step).
 // A launch of its own: in the prologue of every CTA of the next kernel the
@@ -595,7 +598,7 @@ __global__ void __launch_bounds__(BS_NT) k_block_scale(const double *__restrict_
                                                        const int32_t *__restrict__ blk_ptr,
                                                        const double *__restrict__ eps, double inner_tol, int step,
                                                        R *__restrict__ scale, int *__restrict__ inner_state,
-                                                       int *__restrict__ err) {
+                                                       int *__restrict__ inner_steps, int *__restrict__ err) {
     __shared__ double red[BS_NT / 32][3];
     const int blk = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_enter();
@@ -632,7 +635,8 @@ __global__ void __launch_bounds__(BS_NT) k_block_scale(const double *__restrict_
         const double nrm = sqrt(a);
         if (!isfinite(nrm)) atomicOr(err, ERR_NONFINITE);
         scale[blk] = (R)((nrm > eps[blk]) ? eps[blk] / nrm : 1.0);
-        if (test && inner_state[blk] == 0 && sqrt(d) <= inner_tol * sqrt(n)) inner_state[blk] = step;
+        if (test && inner_state[blk] == 0 && inner_steps[blk] != 0 && sqrt(d) <= inner_tol * sqrt(n))
+            inner_state[blk] = inner_steps[blk] = step;
     }
 }
 
@@ -660,76 +664,102 @@ __global__ void k_block_norms(const double *__restrict__ partials, const int32_t
 }
 
 // ----------------------------------------------------------------- gridding
-// Per warp, in rounds of 32 visibilities of its slice of the chunk: phase 1
-// (lane per visibility) forms Theta v, the 8 products w0[a] Theta v and the 8
-// weights w1[b] into the warp's staging area; phase 2 (the warp per
-// visibility) adds the 8 x 8 footprint w1[b] (w0[a] Theta v) into the warp's
-// private (T+8)^2 tile.  Finally the CTA sums the private tiles in warp order
-// and writes the chunk's partial tile.  GR_DUAL fuses the
-// end of the data step: p = P_B(w) = y + c (w - y), v = U (z - p).
-// Lane l of the scattering warp owns footprint column l mod 8 of rows l/8
-// and l/8 + 4; with the private-tile pitch T + 8 = 8 mod 16 (in 8-byte
-// words) the two rows a half-warp touches fall in disjoint bank halves, so
-// the read-modify-write of the tile is free of bank conflicts.
-constexpr int GRID_MINV = 16;   // least visibilities per scattering warp
-// NW warps per CTA (4 or 8; FP64: 4): eight split a chunk finer, four
+// A work item is a sequence of groups (up to 32 visibilities of one block) of
+// one tile; a warp or the NW warps of a CTA add its footprints into a private
+// (T+8)^2 tile per warp, and the sum of the private tiles is the item's
+// partial tile.  Per group: each lane stages one visibility (dual update,
+// Theta v, the 8 products w0[a] Theta v and the 8 weights w1[b]) in the warp's
+// staging area, then the warp adds the footprints one after the other, each
+// lane accumulating two cells in registers (columns b and b + 4 of row a =
+// lane / 4: 16 staged bytes a lane and visibility, 20 with two rows of a
+// column) and adding them to the tile when the base cell changes (the order
+// keeps visibilities of one cell together).  GR_DUAL fuses the end of the data step: p = P_B(w) = y + c (w - y), v = U (z - p).
+//
+// Items of up to `small` groups take one warp, NW of them share a CTA that
+// has no CTA barrier; larger ones are spread over the warps of a CTA.  An
+// item of one block and a CTA per item left most warps idle (4096^2, 8.4M
+// visibilities in 256 blocks: 81k items of 103 on average, 5700
+// instructions each, against 36k of 2 to 32 groups now).  Before -> now: 644 ->
+// 359 us there (and the combine pass, with half the partial tiles, 138 ->
+// 112), 125 -> 111 us at 1024^2 (4.2M visibilities, 64 blocks, dual step), 37
+// -> 29 us at 640 x 480 (700k), 27 -> 28 us at 512^2 (524k).  What bounds it
+// now: issue slots (71 % busy at 1024^2, 20 instructions a visibility) and
+// the shared-memory path (71 %).
+// With the private-tile pitch T + 8 = 8 mod 16 (in 8-byte words) rows a and a
+// + 2 share banks: lanes of rows 2, 3, 6 and 7 take column b + 4 first.
+// A warp's staging area: per visibility w0[a] Theta v and the pairs (w1[b],
+// w1[b+4]).  The pitch keeps rows 16-byte aligned and the 8 (4) rows that a
+// warp reads at once in distinct banks.
+template <typename R> struct GridStage {
+    static constexpr int PITCH = sizeof(R) == 4 ? 34 : 33;
+    cplx_t<R> p[8][PITCH];
+    cplx_t<R> w[4][PITCH];
+};
+template <typename R, int T> struct __align__(16) GridWarp {
+    cplx_t<R> tile[(T + HALO) * (T + HALO)];
+    GridStage<R> st;
+};
+
+// NW warps per CTA (4 or 8; FP64: 4): eight split an item finer, four
 // leave room for more CTAs per SM (the autotuner picks per problem).
 template <typename R, int T, int MODE, int NW>
-__global__ void __launch_bounds__(NW * 32) k_grid(VisArgs<R> A, cplx_t<R> *__restrict__ gpart) {
+__global__ void __launch_bounds__(NW * 32, sizeof(R) == 8 || T == 32 ? 1 : 28 / NW)
+    k_grid(VisArgs<R> A, int n_large, int n_items,
+                                                  cplx_t<R> *__restrict__ gpart) {
     using C = cplx_t<R>;
-    constexpr int NT = NW * 32;
-    constexpr int E = T + HALO, P = E;   // P: pitch of the private tiles (8 mod 16 words)
+    constexpr int E = T + HALO, P = E, EE = E * E;   // P: pitch of the private tiles (8 mod 16 words)
     static_assert(P % 16 == 8, "private-tile pitch");
+    constexpr int VEC = 16 / sizeof(C), NV = EE / VEC;   // 16-byte pieces of a tile
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    // per-warp staging of 32 visibilities, component-major with a pitch of
-    // 33 so that the stores of a warp's lanes and their reads of one
-    // visibility both hit distinct banks
-    constexpr int SP = 33, SW = 2 * 4 * SP;   // complex words per warp: 4 x SP pairs
-    C *priv = reinterpret_cast<C *>(smem_raw);                          // NW * E * P
-    C *sa_all = priv + NW * E * P;                                      // NW x 4 x SP pairs (w0[a] Theta v, w0[a+4] Theta v)
-    R *sb_all = reinterpret_cast<R *>(sa_all + NW * SW);                // NW x 8 x SP: w1[b]
-
-    // largest chunks first, so that the last wave holds the small ones
-    const int ch = A.ch_order[blockIdx.x];
-    const int start = A.ch_start[ch], count = A.ch_count[ch], tl = A.ch_tile[ch];
-    const int row0 = (tl / A.ntile1) * T, col0 = (tl % A.ntile1) * T;
+    GridWarp<R, T> *W = reinterpret_cast<GridWarp<R, T> *>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int blk = A.ch_block[ch];
-    // warps that scatter: at least GRID_MINV visibilities each, so that a
-    // small chunk clears and sums only as many private tiles as it fills
-    const int nwu = min(NW, max(1, (count + GRID_MINV - 1) / GRID_MINV));
-    for (int e = threadIdx.x; e < nwu * E * P; e += NT) priv[e] = C{0, 0};
+    // largest items first, so that the last wave holds the small ones
+    const bool large = (int)blockIdx.x < n_large;
+    const int pos = large ? (int)blockIdx.x : n_large + ((int)blockIdx.x - n_large) * NW + warp;
+    const int item = pos < n_items ? A.it_order[pos] : -1;
+    const int2 ig = item >= 0 ? A.it_grp[item] : make_int2(0, 0);
+    // warps that share the item, at least two groups each, so that only as
+    // many private tiles are cleared and summed as get filled
+    const int nwu = large ? min(NW, max(1, ig.y / 2)) : 1, w = large ? warp : 0;
+    C *mine = W[warp].tile;
+    if (w < nwu)
+        for (int e = lane; e < NV; e += 32) reinterpret_cast<float4 *>(mine)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
     pdl_enter();
-    // a block outside the active set D keeps v_j, so its chunks' partial
-    // tiles from the last gridding still hold G^dagger Theta^dagger v_j
-    const bool act = MODE != GR_DUAL || !A.bmask || A.bmask[blk];
-    if (!act && !(A.regrid && *A.regrid)) return;
-    R c = 0;
-    // Algorithm 2 stopped early (stopping test): the prox output is the p
-    // the stopping step kept, not P_B of the current w
-    bool done = false;
-    if (MODE == GR_DUAL && act) {
-        const int stopped = A.inner_tol > 0 && A.n_itr > 1 ? A.inner_state[blk] : 0;
-        done = stopped != 0;
-        c = A.scale[blk];
-        if (threadIdx.x == 0 && A.inner_steps) A.inner_steps[blk] = done ? stopped : A.n_itr;
+    if (item < 0) return;
+    // blocks outside the active set D keep v_j: an item with none inside
+    // keeps its partial tile of the last gridding, unless that may be stale
+    if (MODE == GR_DUAL && A.bmask && !*A.regrid) {
+        bool any = false;
+        for (int g = lane; g < ig.y; g += 32) any = any || A.bmask[A.gg[ig.x + g].w];
+        if (!__any_sync(0xffffffffu, any)) return;   // (the same for every warp of the item)
     }
-    if (MODE == GR_DUAL && act && A.seen && threadIdx.x == 0) A.seen[blk] = 1;
-    __syncthreads();
-
-    C *mine = priv + warp * E * P;
-    const int bcol = lane & 7, a0 = lane >> 3;   // rows a0 and a0 + 4
-    // a lane's visibility of the current round, loaded one round ahead so
-    // that the loads of round r + 1 are in flight during the scatter of r
+    const int arow = lane >> 2, bcol = lane & 3;   // row, and columns bcol and bcol + 4
+    const bool swap = arow & 2;
     struct In {
         VisRec<R> rc;
         C a, b, z;   // GR_DUAL active: y, w, z (stopped early: p, -, z); inactive: v; operator modes: input
         R th;
     };
-    auto load_in = [&](int gi, In &o) {
+    // of a group's block: inside D, Algorithm 2 stopped early (stopping
+    // test: the prox output is the p the stopping step kept, not P_B of the
+    // current w), the P_B scale
+    struct Blk {
+        bool act, done;
+        R c;
+    };
+    auto block_of = [&](int blk) {
+        Blk o{true, false, R(0)};
+        if (MODE == GR_DUAL) {
+            o.act = !A.bmask || A.bmask[blk];
+            if (A.tol_on) o.done = A.inner_state[blk] != 0;
+            o.c = A.scale[blk];
+        }
+        return o;
+    };
+    auto load_in = [&](int gi, const Blk &q, In &o) {
         o.rc = A.rec[gi];
-        if (MODE == GR_DUAL && act) {
-            if (done) {
+        if (MODE == GR_DUAL && q.act) {
+            if (q.done) {
                 o.a = A.p[gi];
             } else {
                 o.a = A.y[gi];
@@ -743,134 +773,124 @@ __global__ void __launch_bounds__(NW * 32) k_grid(VisArgs<R> A, cplx_t<R> *__res
         }
         o.th = A.theta_v ? A.theta_v[gi] : A.theta_s;
     };
-    // warp w owns a contiguous slice of the chunk (the sort order makes runs
-    // of visibilities share a first tap) and works through it in rounds of
-    // 32: each lane stages one visibility (dual update, Theta v, weights) in
-    // the warp's staging area, then the warp adds the 32 footprints one after
-    // the other, each lane accumulating its two cells in registers and
-    // writing the private tile only when the base cell changes.  Warps never
-    // wait for one another inside the loop.
-    C *sa = sa_all + warp * SW;
-    R *sb = sb_all + warp * KB_J * SP;
-    const int seg = (count + nwu - 1) / nwu;
-    const int v0 = warp < nwu ? min(count, warp * seg) : count, v1 = min(count, v0 + seg);
-    In cur;
-    if (v0 + lane < v1) load_in(start + v0 + lane, cur);
-    int run = -1;   // base cell (packed local row | col << 16) of the run being accumulated
-    C acc0{0, 0}, acc1{0, 0};
-    auto fetch = [&](int i, C &pa, C &pb, R &wb) {   // w0[a0] Theta v, w0[a0+4] Theta v, w1[bcol]
-        if constexpr (sizeof(R) == 4) {
-            const float4 q = *reinterpret_cast<const float4 *>(sa + 2 * (a0 * SP + i));
-            pa = C{q.x, q.y};
-            pb = C{q.z, q.w};
-        } else {
-            pa = sa[2 * (a0 * SP + i)];
-            pb = sa[2 * (a0 * SP + i) + 1];
-        }
-        wb = sb[bcol * SP + i];
-    };
-    auto accumulate = [&](const C &pa, const C &pb, R wb) {
-        acc0.x += wb * pa.x;
-        acc0.y += wb * pa.y;
-        acc1.x += wb * pb.x;
-        acc1.y += wb * pb.y;
-    };
-    auto flush = [&]() {   // add the run's two cells of this lane into the private tile
-        C *cell = mine + ((run & 0xffff) + a0) * P + (run >> 16) + bcol;
-        const C g0 = cell[0], g1 = cell[4 * P];
-        cell[0] = cadd(g0, acc0);
-        cell[4 * P] = cadd(g1, acc1);
-    };
-    for (int base = v0; base < v1; base += 32) {
-        const int n = min(32, v1 - base);
-        int mylb = -1;
-        if (lane < n) {
-            const int gi = start + base + lane;
-            const VisRec<R> rc = cur.rc;
-            C vv;
-            if (MODE == GR_DUAL && act) {
-                const C zz = cur.z;
-                C pp;
-                if (done) {
-                    pp = cur.a;
-                } else {
-                    const C yy = cur.a, ww = cur.b;
-                    pp = C{yy.x + c * (ww.x - yy.x), yy.y + c * (ww.y - yy.y)};
-                    A.p[gi] = pp;
+    GridStage<R> &st = W[warp].st;
+    const int g0 = ig.x + (w < nwu ? w * ig.y / nwu : 0), g1 = ig.x + (w < nwu ? (w + 1) * ig.y / nwu : 0);
+    if (g0 < g1) {
+        int4 D = A.gg[g0], Dn = g0 + 1 < g1 ? A.gg[g0 + 1] : D;   // this group and the next
+        Blk bk = block_of(D.w);
+        In cur;
+        if (lane < D.y) load_in(D.x + lane, bk, cur);
+        const int row0 = (D.z / A.ntile1) * T, col0 = (D.z % A.ntile1) * T;
+        C *cells0 = mine + arow * P + bcol + (swap ? 4 : 0), *cells1 = mine + arow * P + bcol + (swap ? 0 : 4);
+        int run = -1;   // base cell (tile offset) of the run being accumulated
+        C acc0{0, 0}, acc1{0, 0};   // columns bcol, bcol + 4
+        auto flush = [&]() {   // add the run's two cells of this lane into the private tile
+            const C t0 = cells0[run], t1 = cells1[run];
+            cells0[run] = cadd(t0, swap ? acc1 : acc0);
+            cells1[run] = cadd(t1, swap ? acc0 : acc1);
+        };
+        auto accumulate = [&](C w, C q) {
+            acc0.x += w.x * q.x;
+            acc0.y += w.x * q.y;
+            acc1.x += w.y * q.x;
+            acc1.y += w.y * q.y;
+        };
+        for (int g = g0; g < g1; ++g) {
+            const int n = D.y;
+            int mylb = -1;
+            R w0[KB_J] = {}, w1[KB_J] = {};
+            C tv{0, 0};
+            if (lane < n) {
+                const int gi = D.x + lane;
+                const VisRec<R> rc = cur.rc;
+                C vv = cur.a;
+                if (MODE == GR_DUAL && bk.act) {
+                    C pp = cur.a;
+                    if (!bk.done) {
+                        pp = C{cur.a.x + bk.c * (cur.b.x - cur.a.x), cur.a.y + bk.c * (cur.b.y - cur.a.y)};
+                        A.p[gi] = pp;
+                    }
+                    vv = C{rc.U * (cur.z.x - pp.x), rc.U * (cur.z.y - pp.y)};
+                    A.v[gi] = vv;
+                } else if (MODE == GR_OP_U) {
+                    vv = C{rc.U * vv.x, rc.U * vv.y};
                 }
-                vv = C{rc.U * (zz.x - pp.x), rc.U * (zz.y - pp.y)};
-                A.v[gi] = vv;
-            } else if (MODE == GR_DUAL) {
-                vv = cur.a;
-            } else {
-                vv = cur.a;
-                if (MODE == GR_OP_U) vv = C{rc.U * vv.x, rc.U * vv.y};
+                tv = C{cur.th * vv.x, cur.th * vv.y};
+                kb_weights(rc.f0, w0, A);
+                kb_weights(rc.f1, w1, A);
+                mylb = ((rc.packed & 0xffff) - row0) * P + ((rc.packed >> 16) & 0xffff) - col0;
             }
-            const R th = cur.th;
-            const C tv{th * vv.x, th * vv.y};
-            R w0[KB_J], w1[KB_J];
-            kb_weights(rc.f0, w0, A);
-            kb_weights(rc.f1, w1, A);
+            // (lanes past the group stage zeros: the loop below works in fours)
 #pragma unroll
-            for (int a = 0; a < KB_J / 2; ++a) {   // lane rows (a, a+4) read one pair
-                C *da = sa + 2 * (a * SP + lane);
-                if constexpr (sizeof(R) == 4) {
-                    *reinterpret_cast<float4 *>(da) =
-                        make_float4(w0[a] * tv.x, w0[a] * tv.y, w0[a + 4] * tv.x, w0[a + 4] * tv.y);
+            for (int a = 0; a < KB_J; ++a) st.p[a][lane] = C{w0[a] * tv.x, w0[a] * tv.y};
+#pragma unroll
+            for (int j = 0; j < KB_J / 2; ++j) st.w[j][lane] = C{w1[j], w1[j + 4]};
+            if (MODE == GR_DUAL && A.seen && lane == 0 && bk.act && !A.seen[D.w]) A.seen[D.w] = 1;
+            // the group's visibilities that start a new run: lane 0 compares
+            // with the run carried over
+            const int prev = __shfl_up_sync(0xffffffffu, mylb, 1);
+            const unsigned starts = __ballot_sync(0xffffffffu, lane < n && mylb != (lane == 0 ? run : prev));
+            __syncwarp();
+            if (g + 1 < g1) {   // the next group, in flight during the sums
+                D = Dn;
+                bk = block_of(D.w);
+                if (lane < D.y) load_in(D.x + lane, bk, cur);
+                if (g + 2 < g1) Dn = A.gg[g + 2];
+            }
+            for (int i = 0; i < n; i += 4) {
+                C pq[4], wq[4];
+                if constexpr (sizeof(R) == 4) {   // two visibilities per 16-byte read
+#pragma unroll
+                    for (int q = 0; q < 4; q += 2) {
+                        const float4 u = *reinterpret_cast<const float4 *>(&st.p[arow][i + q]);
+                        const float4 v = *reinterpret_cast<const float4 *>(&st.w[bcol][i + q]);
+                        pq[q] = C{u.x, u.y};
+                        pq[q + 1] = C{u.z, u.w};
+                        wq[q] = C{v.x, v.y};
+                        wq[q + 1] = C{v.z, v.w};
+                    }
                 } else {
-                    da[0] = C{w0[a] * tv.x, w0[a] * tv.y};
-                    da[1] = C{w0[a + 4] * tv.x, w0[a + 4] * tv.y};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        pq[q] = st.p[arow][i + q];
+                        wq[q] = st.w[bcol][i + q];
+                    }
+                }
+                const unsigned m = (starts >> i) & 15u;
+                if (m == 0) {   // (m is uniform across the warp)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) accumulate(wq[q], pq[q]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (m & (1u << q)) {
+                            if (run >= 0) flush();
+                            run = __shfl_sync(0xffffffffu, mylb, i + q);
+                            acc0 = acc1 = C{0, 0};
+                        }
+                        accumulate(wq[q], pq[q]);
+                    }
                 }
             }
-#pragma unroll
-            for (int j = 0; j < KB_J; ++j) sb[j * SP + lane] = w1[j];
-            mylb = ((rc.packed & 0xffff) - row0) | ((((rc.packed >> 16) & 0xffff) - col0) << 16);
+            __syncwarp();   // the staging is rewritten by the next group
         }
-        // the visibilities of the round that start a new run (the order is
-        // sorted by base cell): lane 0 compares with the run carried over
-        const int prev = __shfl_up_sync(0xffffffffu, mylb, 1);
-        unsigned starts = __ballot_sync(0xffffffffu, lane < n && mylb != (lane == 0 ? run : prev));
-        __syncwarp();
-        if (base + 32 + lane < v1) load_in(start + base + 32 + lane, cur);   // next round, in flight during the scatter
-        // the warp walks the round run by run (uniform control flow): at a
-        // run start the finished run is added to the tile, inside a run the
-        // footprints accumulate in registers, four at a time
-        int i = 0;
-        while (i < n) {
-            const int e = starts ? __ffs(starts) - 1 : n;
-            if (e == i) {
-                if (run >= 0) flush();
-                run = __shfl_sync(0xffffffffu, mylb, i);
-                acc0 = C{0, 0};
-                acc1 = C{0, 0};
-                starts &= starts - 1;
-                continue;
-            }
-            for (; i + 4 <= e; i += 4) {
-                C pa[4], pb[4];
-                R wb[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) fetch(i + q, pa[q], pb[q], wb[q]);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) accumulate(pa[q], pb[q], wb[q]);
-            }
-            for (; i < e; ++i) {
-                C pa, pb;
-                R wb;
-                fetch(i, pa, pb, wb);
-                accumulate(pa, pb, wb);
-            }
-        }
-        __syncwarp();   // the staging is rewritten by the next round
+        if (run >= 0) flush();
     }
-    if (run >= 0) flush();
+    float4 *out = reinterpret_cast<float4 *>(gpart + (int64_t)item * EE);
+    if (!large) {
+        __syncwarp();
+        for (int e = lane; e < NV; e += 32) out[e] = reinterpret_cast<const float4 *>(mine)[e];
+        return;
+    }
     __syncthreads();
-    C *out = gpart + (int64_t)ch * E * E;
-    for (int e = threadIdx.x; e < E * E; e += NT) {
-        const int r = e / E, cc = e % E;
-        C s{0, 0};
-        for (int k = 0; k < nwu; ++k) s = cadd(s, priv[k * E * P + r * P + cc]);
-        out[e] = s;
+    for (int e = threadIdx.x; e < NV; e += NW * 32) {
+        C s[VEC];
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) s[q] = W[0].tile[e * VEC + q];
+        for (int k = 1; k < nwu; ++k)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) s[q] = cadd(s[q], W[k].tile[e * VEC + q]);
+        out[e] = *reinterpret_cast<const float4 *>(s);
     }
 }
 
@@ -932,11 +952,9 @@ template <typename R> VisArgs<R> make_args(ppd_ctx *c) {
     A.rec = static_cast<const VisRec<R> *>(c->rec);
     A.theta_v = static_cast<const R *>(c->theta_v);
     A.theta_s = (R)c->theta_scalar;
-    A.ch_start = c->ch.start;
-    A.ch_count = c->ch.count;
-    A.ch_tile = c->ch.tile;
-    A.ch_block = c->ch.block;
-    A.ch_order = c->ch.order;
+    A.gg = c->ch.gg;
+    A.it_grp = c->ch.it_grp;
+    A.it_order = c->ch.order;
     A.K0 = c->K0;
     A.K1 = c->K1;
     A.ntile1 = c->K1 / c->T;
@@ -963,18 +981,12 @@ template <typename R> VisArgs<R> make_args(ppd_ctx *c) {
     A.bmask = c->rand_on ? c->mask_cur : nullptr;
     A.seen = c->rand_on ? c->blk_seen : nullptr;
     A.regrid = c->rand_on ? c->regrid_d : nullptr;
-    A.inner_tol = c->cfg.inner_tol;
+    A.tol_on = c->cfg.inner_tol > 0;
     A.step = c->next_step;
     A.n_itr = c->cfg.n_itr;
     A.inner_state = c->inner_state;
     A.inner_steps = c->inner_steps;
     return A;
-}
-
-template <typename R, int T, int NW> size_t grid_smem() {
-    constexpr int E = T + HALO, P = E, SP = 33;
-    return (size_t)NW * E * P * sizeof(cplx_t<R>) + (size_t)NW * 8 * SP * sizeof(cplx_t<R>) +
-           (size_t)NW * KB_J * SP * sizeof(R);
 }
 
 // the blocks' scales from the norm partials of the kernel before
@@ -983,7 +995,7 @@ template <typename R> int block_scales(ppd_ctx *c, int step, cudaStream_t s) {
     PPD_CHECK(launch_begin(c, "block_scale", s, &site));
     launch(c, true, k_block_scale<R>, (unsigned)c->d, BS_NT, 0, s, (const double *)c->partials,
            (const int32_t *)c->ch.blk_ptr, (const double *)c->eps_d, c->cfg.inner_tol, step,
-           static_cast<R *>(c->scale), c->inner_state, c->err);
+           static_cast<R *>(c->scale), c->inner_state, c->inner_steps, c->err);
     return launch_end(c, site, s);
 }
 
@@ -1012,7 +1024,7 @@ int degrid_t(ppd_ctx *c, int mode, const cplx_t<R> *grid, cplx_t<R> *out, const 
 }
 
 template <typename R, int T, int NW> int grid_launch(ppd_ctx *c, int mode, const VisArgs<R> &A, cudaStream_t s) {
-    const size_t sh = grid_smem<R, T, NW>();
+    const size_t sh = NW * sizeof(GridWarp<R, T>);
     PPD_CHECK(smem_attr((const void *)k_grid<R, T, GR_OP, NW>, (int)sh));
     PPD_CHECK(smem_attr((const void *)k_grid<R, T, GR_OP_U, NW>, (int)sh));
     PPD_CHECK(smem_attr((const void *)k_grid<R, T, GR_DUAL, NW>, (int)sh));
@@ -1021,7 +1033,9 @@ template <typename R, int T, int NW> int grid_launch(ppd_ctx *c, int mode, const
     auto k = mode == GR_OP     ? k_grid<R, T, GR_OP, NW>
              : mode == GR_OP_U ? k_grid<R, T, GR_OP_U, NW>
                                : k_grid<R, T, GR_DUAL, NW>;
-    launch(c, true, k, (unsigned)c->ch.n, NW * 32, sh, s, A, static_cast<cplx_t<R> *>(c->gpart));
+    const int64_t small = c->ch.n - c->ch.n_large;
+    launch(c, true, k, (unsigned)(c->ch.n_large + (small + NW - 1) / NW), NW * 32, sh, s, A, (int)c->ch.n_large,
+           (int)c->ch.n, static_cast<cplx_t<R> *>(c->gpart));
     return launch_end(c, site, s);
 }
 
