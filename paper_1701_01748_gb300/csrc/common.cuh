@@ -124,12 +124,15 @@ struct TimingSite {
     cudaEvent_t start, stop;
 };
 
-// Stages of a mixed-radix FFT of length K (radices 2, 3, 4, 5; ns = 0 when
-// K has another prime factor).
+// Stages of a mixed-radix FFT of length K (radices up to 16 with prime
+// factors 2, 3, 5; ns = 0 when K has another prime factor): per stage the
+// radix, the twiddles' step K / (Ns rad) in the table of K, and reciprocals
+// of the span Ns and of K / rad.
 struct FftPlan {
-    static constexpr int MAX_STAGES = 16;
+    static constexpr int MAX_STAGES = 8;
     int K = 0, ns = 0;
-    int rad[MAX_STAGES] = {};
+    int rad[MAX_STAGES] = {}, tstep[MAX_STAGES] = {};
+    uint32_t inv_ns[MAX_STAGES] = {}, inv_m[MAX_STAGES] = {};
 };
 FftPlan make_fft_plan(int K);
 // lengths the FFT passes handle: 32 <= K <= 8192 with prime factors 2, 3, 5
@@ -405,8 +408,8 @@ template <typename R> struct PrimalSums {
         c = (t - s) - y;
         s = t;
     }
-    __device__ __forceinline__ void write(double *part3) const {
-        cta_sum3<256>((double)sd - (double)cd, (double)sx - (double)cx, (double)se - (double)ce, part3);
+    template <int NTH> __device__ __forceinline__ void write(double *part3) const {
+        cta_sum3<NTH>((double)sd - (double)cd, (double)sx - (double)cx, (double)se - (double)ce, part3);
     }
 };
 

@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(NT) k_primal(PrimalArgs<R> P, const R *__restr
     PrimalSums<R> acc;
     for (int64_t e = blockIdx.x * (int64_t)NT + threadIdx.x; e < N; e += (int64_t)gridDim.x * NT)
         primal_pixel(P, e, g[e], acc);
-    acc.write(part + 3 * (int64_t)blockIdx.x);
+    acc.template write<NT>(part + 3 * (int64_t)blockIdx.x);
 }
 
 __global__ void k_reduce3(const double *__restrict__ part, int n, double *__restrict__ out) {
