@@ -894,6 +894,10 @@ __global__ void __launch_bounds__(NW * 32, sizeof(R) == 8 || T == 32 ? 1 : 28 / 
     }
 }
 
+template <int V> struct Count {
+    static constexpr int value = V;
+};
+
 // ----------------------------------------------------------------- combine
 // One CTA per active tile (a tile with chunks, or below/right of one):
 // grid[r][c] = sum of the partial tiles covering the cell, in a fixed order:
@@ -903,47 +907,68 @@ __global__ void __launch_bounds__(NW * 32, sizeof(R) == 8 || T == 32 ? 1 : 28 / 
 // the T x T sums, formed from row-major partial-tile reads, are transposed
 // in shared memory and written as whole column segments.  Tiles never
 // touched by any visibility stay zero from the initial clear.
-template <typename R, int T>
-__global__ void __launch_bounds__(256) k_combine(const cplx_t<R> *__restrict__ gpart,
+//
+// NTH threads per tile read the tile's item ranges themselves, no barrier
+// before the partial tiles.  Where tiles have about one item each, 64 threads
+// with four cells side by side keep four times the loads in flight per
+// thread and as many tiles per SM (4096^2, 36k items: 112 -> 52 us; 960 x 400:
+// 15.6 -> 8.7; 640 x 480: 8.0 -> 6.6); where a tile has several, a thread per
+// cell shortens the sums' chain (1024^2, two items per tile: 64 threads took
+// 20 us, 256 take 15).
+template <typename R, int T, int NTH>
+__global__ void __launch_bounds__(NTH) k_combine(const cplx_t<R> *__restrict__ gpart,
                                                  const int32_t *__restrict__ tile_first,
                                                  const int32_t *__restrict__ tile_n,
                                                  const int32_t *__restrict__ active, int K0, int nt0, int nt1,
                                                  cplx_t<R> *__restrict__ grid) {
     using C = cplx_t<R>;
-    constexpr int E = T + HALO;
-    __shared__ int f_s[4], n_s[4];
+    constexpr int E = T + HALO, CELLS = T * T / NTH;
+    // of a thread's cells the first UPPER lie in the rows above HALO (all or
+    // none when it has one cell)
+    constexpr int UPPER = CELLS == 1 ? 1 : CELLS * HALO / T;
+    static_assert(CELLS == 1 || T * HALO % NTH == 0, "cells split at row HALO");
     __shared__ C tr[T][T + 1];
     const int t = active[blockIdx.x];
     const int t0 = t / nt1, t1 = t - t0 * nt1;
-    if (threadIdx.x < 4) {
-        const int up = (t0 + nt0 - 1) % nt0, left = (t1 + nt1 - 1) % nt1;
-        const int tt = threadIdx.x == 0 ? t : threadIdx.x == 1 ? up * nt1 + t1
-                       : threadIdx.x == 2 ? t0 * nt1 + left : up * nt1 + left;
-        f_s[threadIdx.x] = tile_first[tt];
-        n_s[threadIdx.x] = tile_n[tt];
+    const int up = t0 == 0 ? nt0 - 1 : t0 - 1, left = t1 == 0 ? nt1 - 1 : t1 - 1;
+    const int tt[4] = {t, up * nt1 + t1, t0 * nt1 + left, up * nt1 + left};
+    int f[4], n[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        f[q] = __ldg(tile_first + tt[q]);
+        n[q] = __ldg(tile_n + tt[q]);
     }
-    __syncthreads();
     pdl_enter();
-    for (int e = threadIdx.x; e < T * T; e += 256) {
-        const int lr = e / T, lc = e % T;
-        C acc{0, 0};
+    // cell i of this thread: row lr + i NTH / T, column lc
+    const int lr = threadIdx.x / T, lc = threadIdx.x % T;
+    C acc[CELLS];
+#pragma unroll
+    for (int i = 0; i < CELLS; ++i) acc[i] = C{0, 0};
+    auto add = [&](int q, int off, bool in, auto cells) {   // the items of tile q at offset `off`
+        constexpr int NC = decltype(cells)::value;
+        if (!in) return;
+        const C *p = gpart + (int64_t)f[q] * E * E + off + lr * E + lc;
+        if constexpr (CELLS == 1) {
 #pragma unroll 4
-        for (int k = 0; k < n_s[0]; ++k) acc = cadd(acc, gpart[(int64_t)(f_s[0] + k) * E * E + lr * E + lc]);
-        if (lr < HALO)
-            for (int k = 0; k < n_s[1]; ++k)
-                acc = cadd(acc, gpart[(int64_t)(f_s[1] + k) * E * E + (lr + T) * E + lc]);
-        if (lc < HALO)
-            for (int k = 0; k < n_s[2]; ++k)
-                acc = cadd(acc, gpart[(int64_t)(f_s[2] + k) * E * E + lr * E + lc + T]);
-        if (lr < HALO && lc < HALO)
-            for (int k = 0; k < n_s[3]; ++k)
-                acc = cadd(acc, gpart[(int64_t)(f_s[3] + k) * E * E + (lr + T) * E + lc + T]);
-        tr[lc][lr] = acc;
-    }
+            for (int k = 0; k < n[q]; ++k) acc[0] = cadd(acc[0], p[(int64_t)k * (E * E)]);
+        } else {
+            for (int k = 0; k < n[q]; ++k, p += E * E)
+#pragma unroll
+                for (int i = 0; i < NC; ++i) acc[i] = cadd(acc[i], p[i * (NTH / T) * E]);
+        }
+    };
+    const bool upper = CELLS > 1 || lr < HALO;
+    add(0, 0, true, Count<CELLS>{});
+    add(1, T * E, upper, Count<UPPER>{});
+    add(2, T, lc < HALO, Count<CELLS>{});
+    add(3, T * E + T, upper && lc < HALO, Count<UPPER>{});
+#pragma unroll
+    for (int i = 0; i < CELLS; ++i) tr[lc][lr + i * (NTH / T)] = acc[i];
     __syncthreads();
-    for (int e = threadIdx.x; e < T * T; e += 256) {
-        const int lc = e / T, lr = e % T;
-        grid[(int64_t)(t1 * T + lc) * K0 + t0 * T + lr] = tr[lc][lr];
+#pragma unroll
+    for (int i = 0; i < CELLS; ++i) {
+        const int e = threadIdx.x + i * NTH, oc = e / T, orow = e % T;
+        grid[(int64_t)(t1 * T + oc) * K0 + t0 * T + orow] = tr[oc][orow];
     }
 }
 
@@ -1056,7 +1081,10 @@ int grid_t(ppd_ctx *c, int mode, const cplx_t<R> *in, const int64_t *perm, cplx_
     }
     if (c->ch.n_active == 0 || !combine) return PPD_OK;
     PPD_CHECK(launch_begin(c, "grid_combine", s, &site));
-    launch(c, true, k_combine<R, T>, (unsigned)c->ch.n_active, 256, 0, s, (const cplx_t<R> *)gp,
+    constexpr int few = T == 16 ? 64 : 256, many = T == 16 ? 256 : 1024;
+    const bool sparse = c->ch.n * 5 < c->ch.n_active * 6;   // under 1.2 items per written tile
+    launch(c, true, sparse ? k_combine<R, T, few> : k_combine<R, T, many>, (unsigned)c->ch.n_active,
+           sparse ? few : many, 0, s, (const cplx_t<R> *)gp,
            (const int32_t *)c->ch.tile_first, (const int32_t *)c->ch.tile_n, (const int32_t *)c->ch.active, c->K0,
            c->K0 / T, c->K1 / T, grid);
     return launch_end(c, site, s);
