@@ -143,7 +143,8 @@ template <typename R, int TS> constexpr size_t syn_smem() {
 template <typename R, int F, int TS, int MODE>
 __device__ __forceinline__ void ana_tile(const R *__restrict__ src, int in_pitch, int n0, int n1, int R0, int C0,
                                          R *__restrict__ ll, int last, R *__restrict__ cb,
-                                         const R *__restrict__ wb, int L1, R kappa, R *tin, R *rowf) {
+                                         const R *__restrict__ wb, int L1, R kappa, R *__restrict__ dirac, R *tin,
+                                         R *rowf) {
     using G = AnaGeo<TS>;
     constexpr int EXT = 2 * TS + F - 2, PS = G::PS, NR = TS / PS;
     static_assert(2 * TS * NR % NT == 0, "column tasks");
@@ -205,6 +206,17 @@ __device__ __forceinline__ void ana_tile(const R *__restrict__ src, int in_pitch
     }
     copy_wait<0>();
     __syncthreads();
+    if constexpr (F == 2 && MODE == 0) {
+        // the Dirac basis is the input itself: the shortest filter's CTAs of
+        // level 0 write their part of it (a launch of its own was 3 us at
+        // 256^2 and 9 us at 2048^2)
+        if (dirac)
+            for (int e = threadIdx.x; e < 4 * TS * TS; e += NT) {
+                const int r = e / (2 * TS), c = e % (2 * TS);
+                if (2 * R0 + r < n0 && 2 * C0 + c < n1)
+                    dirac[(int64_t)(2 * R0 + r) * L1 + 2 * C0 + c] = R(1.0 / 3.0) * tin[r * G::PI + c];
+            }
+    }
     // rows: task (row i, PS positions): low halves into column q, high into TS + q
     for (int task = threadIdx.x; task < EXT * NR; task += NT) {
         const int i = task % EXT, q0 = (task / EXT) * PS;
@@ -271,13 +283,15 @@ __device__ __forceinline__ void ana_tile(const R *__restrict__ src, int in_pitch
 //         (MODE 0: c = D x / 3) or clip-updated (1: u = clip(u + D x / 3, kappa);
 //         2: u = clip(u + w D x / 3, kappa), w the prior weights wgt, laid out
 //         like coef)
+//   dirac: MODE 0, level 0: the Dirac basis's coefficients x / 3, or null
 //   pmask: active set P of Algorithm 3 (9 flags, Dirac first) or null; in
 //         modes 1 and 2 a basis outside P keeps u_b and is skipped at every level
 template <typename R, int TS, int MODE>
 __global__ void __launch_bounds__(NT) k_sara_ana(const R *__restrict__ in, int in_pitch, int64_t in_bstride, int n0,
                                                  int n1, R *__restrict__ ll, int64_t ll_bstride, int last,
                                                  R *__restrict__ coef, const R *__restrict__ wgt, int L1, int64_t N,
-                                                 R kappa, const uint8_t *__restrict__ pmask) {
+                                                 R kappa, R *__restrict__ dirac,
+                                                 const uint8_t *__restrict__ pmask) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R *tin = reinterpret_cast<R *>(smem_raw), *rowf = tin + AnaGeo<TS>::EXT * AnaGeo<TS>::PI;
     const int b = N_WAVELETS - 1 - blockIdx.y;
@@ -289,7 +303,7 @@ __global__ void __launch_bounds__(NT) k_sara_ana(const R *__restrict__ in, int i
     R *lb = ll + (int64_t)b * ll_bstride;
     R *cb = coef + (int64_t)(b + 1) * N;
     const R *wb = MODE == 2 ? wgt + (int64_t)(b + 1) * N : nullptr;
-#define PPD_ANA(F) ana_tile<R, F, TS, MODE>(src, in_pitch, n0, n1, R0, C0, lb, last, cb, wb, L1, kappa, tin, rowf)
+#define PPD_ANA(F) ana_tile<R, F, TS, MODE>(src, in_pitch, n0, n1, R0, C0, lb, last, cb, wb, L1, kappa, dirac, tin, rowf)
     switch (b) {
         case 0: PPD_ANA(2); break;
         case 1: PPD_ANA(4); break;
@@ -559,11 +573,6 @@ __global__ void __cluster_dims__(N_WAVELETS, 1, 1) __launch_bounds__(NT)
     cluster_sync();   // the peers have read this CTA's samples
 }
 
-template <typename R> __global__ void k_scale_copy(const R *__restrict__ in, R *__restrict__ out, int64_t n, R a) {
-    for (int64_t e = blockIdx.x * (int64_t)NT + threadIdx.x; e < n; e += (int64_t)gridDim.x * NT) out[e] = a * in[e];
-}
-
-inline unsigned nblk(int64_t work) { return (unsigned)std::min<int64_t>((work + NT - 1) / NT, 152 * 8); }
 // tiles of ts x ts quadrant positions covering an h0 x h1 quadrant
 inline unsigned tiles(int h0, int h1, int ts) { return (unsigned)(((h0 + ts - 1) / ts) * ((h1 + ts - 1) / ts)); }
 
@@ -598,7 +607,8 @@ template <typename R> int analysis_all(ppd_ctx *c, const R *x, R *coef, int mode
             PPD_CHECK(smem_attr((const void *)k, (int)ana_smem<R, TS>()));
             PPD_CHECK(launch_begin(c, "sara_analysis", s, &site));
             launch(c, l > 0, k, dim3(tiles(n0 / 2, n1 / 2, TS), N_WAVELETS), NT, ana_smem<R, TS>(), s, in, pitch,
-                   bstride, n0, n1, ll[l & 1], ll_stride, (int)last, coef, wgt, L1, N, alpha, pmask);
+                   bstride, n0, n1, ll[l & 1], ll_stride, (int)last, coef, wgt, L1, N, alpha,
+                   mode == 0 && l == 0 ? coef : nullptr, pmask);
             return launch_end(c, site, s);
         };
         PPD_CHECK(large_tile<R>(tiles(n0 / 2, n1 / 2, 32) * N_WAVELETS) ? go(Int<32>{}) : go(Int<16>{}));
@@ -749,10 +759,6 @@ int make_filters(ppd_ctx *c) {
 }
 
 template <typename R> int psi_analysis(ppd_ctx *c, const R *x, R *coef, cudaStream_t s) {
-    int site;
-    PPD_CHECK(launch_begin(c, "sara_dirac", s, &site));
-    k_scale_copy<R><<<nblk(c->N), NT, 0, s>>>(x, coef, c->N, R(1.0 / 3.0));
-    PPD_CHECK(launch_end(c, site, s));
     return analysis_all<R>(c, x, coef, 0, s);
 }
 
