@@ -1031,18 +1031,16 @@ int degrid_t(ppd_ctx *c, int mode, const cplx_t<R> *grid, cplx_t<R> *out, const 
     A.perm = perm;
     constexpr int E = T + HALO;
     const size_t sh = (size_t)(NTD / 32) * dg_bufs<T>() * E * E * sizeof(cplx_t<R>);
-    PPD_CHECK(smem_attr((const void *)k_degrid<R, T, DG_OP, NTD>, (int)sh));
-    PPD_CHECK(smem_attr((const void *)k_degrid<R, T, DG_DUAL, NTD>, (int)sh));
-    PPD_CHECK(smem_attr((const void *)k_degrid<R, T, DG_FIRST, NTD>, (int)sh));
     const int use_tma = (c->tma_ok && grid == c->grid_a) ? 1 : 0;
     if (c->ch.n_grp == 0) return PPD_OK;
     const unsigned nb = (unsigned)((c->ch.n_warps + NTD / 32 - 1) / (NTD / 32));
-    int site;
-    PPD_CHECK(launch_begin(c, mode == DG_OP ? "degrid_op" : "degrid_dual", s, &site));
-    const long long sf = c->wait_first;
     auto k = mode == DG_OP     ? k_degrid<R, T, DG_OP, NTD>
              : mode == DG_DUAL ? k_degrid<R, T, DG_DUAL, NTD>
                                : k_degrid<R, T, DG_FIRST, NTD>;
+    PPD_CHECK(smem_attr((const void *)k, (int)sh));
+    int site;
+    PPD_CHECK(launch_begin(c, mode == DG_OP ? "degrid_op" : "degrid_dual", s, &site));
+    const long long sf = c->wait_first;
     launch(c, true, k, nb, NTD, sh, s, c->tmap_a, use_tma, grid, A, sf);
     PPD_CHECK(launch_end(c, site, s));
     return mode == DG_OP ? PPD_OK : block_scales<R>(c, 0, s);
@@ -1050,14 +1048,12 @@ int degrid_t(ppd_ctx *c, int mode, const cplx_t<R> *grid, cplx_t<R> *out, const 
 
 template <typename R, int T, int NW> int grid_launch(ppd_ctx *c, int mode, const VisArgs<R> &A, cudaStream_t s) {
     const size_t sh = NW * sizeof(GridWarp<R, T>);
-    PPD_CHECK(smem_attr((const void *)k_grid<R, T, GR_OP, NW>, (int)sh));
-    PPD_CHECK(smem_attr((const void *)k_grid<R, T, GR_OP_U, NW>, (int)sh));
-    PPD_CHECK(smem_attr((const void *)k_grid<R, T, GR_DUAL, NW>, (int)sh));
-    int site;
-    PPD_CHECK(launch_begin(c, mode == GR_DUAL ? "grid_dual" : "grid_op", s, &site));
     auto k = mode == GR_OP     ? k_grid<R, T, GR_OP, NW>
              : mode == GR_OP_U ? k_grid<R, T, GR_OP_U, NW>
                                : k_grid<R, T, GR_DUAL, NW>;
+    PPD_CHECK(smem_attr((const void *)k, (int)sh));
+    int site;
+    PPD_CHECK(launch_begin(c, mode == GR_DUAL ? "grid_dual" : "grid_op", s, &site));
     const int64_t small = c->ch.n - c->ch.n_large;
     launch(c, true, k, (unsigned)(c->ch.n_large + (small + NW - 1) / NW), NW * 32, sh, s, A, (int)c->ch.n_large,
            (int)c->ch.n, static_cast<cplx_t<R> *>(c->gpart));
