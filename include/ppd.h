@@ -161,7 +161,7 @@ typedef struct {
     int32_t  K0, K1;            /* oversampled grid */
     int32_t  tile;              /* gridding tile side */
     int32_t  chunk;             /* max visibilities per work item */
-    int64_t  n_chunks;          /* gridding work items */
+    int64_t  n_chunks;          /* runs of at most chunk visibilities of one tile and block */
     int64_t  M;                 /* visibilities */
     double   convergence_lhs;   /* tau*zeta*||Psi W||^2 + tau*eta*||U^{1/2}Phi||^2 (Eq. "convergence-req-explicit-pd"), < 1 */
     double   psiw_norm_sq;      /* ||Psi W||_S^2 of the prior weights (1 when W = I) */
@@ -348,8 +348,8 @@ PPD_API void ppd_group_destroy(ppd_group *g);
  * fixed device-memory budget reserved at start-up or real-time loops that must
  * not block on the allocator or meet an out-of-memory error mid-way.  The
  * paper has no counterpart; this is a deployment variant of the operator.
- * The gridding scratch (one (T+8)^2 complex tile per work item, see
- * ppd_params.n_chunks) comes from one fixed device array of
+ * The gridding scratch (at most one (T+8)^2 complex tile per
+ * ppd_params.n_chunks, the size that is checked) comes from one fixed device array of
  * PPD_NOALLOC_SCRATCH_BYTES that the library holds on every GPU it is loaded
  * on until the process exits.  The call runs on the context's device (see
  * the conventions above) and uses that device's copy of the array.  The

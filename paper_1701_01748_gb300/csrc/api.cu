@@ -881,7 +881,6 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     std::vector<int32_t> tfirst(ntiles, 0), tn(ntiles, 0), in;
     std::vector<int4> grp;
     std::vector<int2> it;
-    const int gsz = std::min(32, c->C);
     int64_t n_tb = 0;
     for (int64_t i = 0; i < M;) {
         const uint64_t k0 = key[c->perm_h[i]];
@@ -890,22 +889,25 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
         while (j < M && key[c->perm_h[j]] / KK == tb) ++j;
         const int tile = (int)(tb / (uint64_t)c->d), blk = (int)(tb % (uint64_t)c->d);
         n_tb += (j - i + c->C - 1) / c->C;
-        for (int64_t s = i; s < j; s += gsz) {
-            const int n = (int)std::min<int64_t>(gsz, j - s);
-            if (tn[tile] == 0 || in.back() + n > c->C) {
+        // a group ends where its item is full, so that a tile has at most as
+        // many items as runs of C visibilities of one block (n_tb)
+        for (int64_t s = i; s < j;) {
+            if (tn[tile] == 0 || in.back() == c->C) {
                 if (tn[tile]++ == 0) tfirst[tile] = (int32_t)it.size();
                 it.push_back(make_int2((int)grp.size(), 0));
                 in.push_back(0);
             }
+            const int n = (int)std::min<int64_t>(std::min(32, c->C - in.back()), j - s);
             it.back().y++;
             in.back() += n;
             grp.push_back(make_int4((int)s, n, tile, blk));
+            s += n;
         }
         i = j;
     }
     const int64_t nch = (int64_t)it.size();
     const std::vector<int4> gg = grp;   // (the degridding's copy is reordered below)
-    // tiles the gridding can reach: a tile with chunks and the tiles below,
+    // tiles the gridding can reach: a tile with items and the tiles below,
     // right and below-right of it (the extended footprint's halo)
     std::vector<int32_t> active;
     {
@@ -920,7 +922,7 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
         for (int t = 0; t < ntiles; ++t)
             if (mark[t]) active.push_back(t);
     }
-    // FFT pruning: rows/columns the degridding reads (tiles with chunks plus
+    // FFT pruning: rows/columns the degridding reads (tiles with items plus
     // their halo) and rows/columns the gridding can write (active tiles)
     std::vector<char> rf(c->K0, 0), cf(c->K1, 0), ri(c->K0, 0), ci(c->K1, 0);
     {
@@ -997,8 +999,8 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     c->ch.n_warps = (int32_t)nwarps;
     c->ch.n_runs = nruns;
     // default gridding CTA shape (unless configured or autotuned): eight
-    // warps while the chunks make few waves, four (more CTAs per SM) beyond
-    // twelve chunks per SM
+    // warps while the items make few waves, four (more CTAs per SM) beyond
+    // twelve items per SM
     if (c->cfg.grid_warps == 0 && !c->shape_tuned && c->is_f32) {
         c->grid_nw = nch > 12LL * std::max(sms, 1) ? 4 : 8;
     }

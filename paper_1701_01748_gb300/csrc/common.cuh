@@ -47,7 +47,7 @@ constexpr int HALO = 8;          // extended tile = (T + HALO)^2 cells
 constexpr int N_BASES = 9;       // Dirac + db1..db8
 constexpr int N_WAVELETS = 8;
 constexpr int MAX_TAPS = 16;     // db8
-// per-chunk norm partials: ||w-y||^2, ||Theta q - y||^2 and, for the
+// per-run norm partials: ||w-y||^2, ||Theta q - y||^2 and, for the
 // Algorithm 2 stopping test, ||zbar^t - zbar^(t-1)||^2, ||zbar^t||^2
 constexpr int NPART = 4;
 constexpr double INV_TWO_PI = 0.15915494309189535;
@@ -153,9 +153,9 @@ struct Chunks {
     int32_t *tile_first = nullptr, *tile_n = nullptr;                                // device, n_tiles
     // work of the degridding and sub-iterations: groups of at most 32
     // visibilities of one tile and block {start, count, tile, block}, shared
-    // out equally to n_warps warps (warp w: warp_grp[w] .. warp_grp[w+1] - 1); a warp's maximal sequences
-    // of groups of one block are its runs (warp w: warp_run[w] ..
-    // warp_run[w+1] - 1); run r writes its norm partials to slot
+    // out equally to n_warps warps (warp w: warp_grp[w] .. warp_grp[w+1] - 1);
+    // a warp's maximal sequences of groups of one block are its runs (warp w:
+    // warp_run[w] .. warp_run[w+1] - 1); run r writes its norm partials to slot
     // run_pos[r], block b owns slots blk_ptr[b] .. blk_ptr[b+1] - 1
     int32_t n_grp = 0, n_warps = 0;
     int64_t n_runs = 0;
@@ -233,7 +233,7 @@ struct ppd_ctx {
     int *stop_flag = nullptr;                          // global stopping rule (device, 1 int)
     cudaStream_t stream2 = nullptr;                   // prior (SARA) branch of the iteration
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    void *gpart = nullptr;           // n_chunks x (T+HALO)^2 complex
+    void *gpart = nullptr;           // items x (T+HALO)^2 complex
     int *err = nullptr;              // device error word
     long long wait_first = ppd::SPIN_LIMIT;   // polls of the degridding's first TMA wait (ppd_set_wait_limit)
     CUtensorMap tmap_a;              // TMA descriptor of grid_a

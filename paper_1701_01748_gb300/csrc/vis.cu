@@ -10,11 +10,12 @@
 //    summed across work items in a fixed order (deterministic, no atomics)
 //
 // Work decomposition: visibilities are sorted by (tile of the centred grid
-// holding the first tap, block, base cell); a "chunk" is a run of at most C
-// visibilities of one tile and one block, and each CTA owns one chunk.  The
-// CTA stages the (T+8) x (T+8) extended grid tile in shared memory (TMA for
-// interior tiles, wrapped plain loads at the grid edge) for degridding, or
-// accumulates into it for gridding.
+// holding the first tap, block, base cell) and cut into groups of at most 32
+// of one tile and block.  Degridding and sub-iterations share the groups out
+// to warps; a degridding warp stages the (T+8) x (T+8) extended grid tile of
+// its groups in shared memory (TMA for interior tiles, wrapped plain loads at
+// the grid edge).  Gridding work items are sequences of groups of one tile; a
+// warp or a CTA accumulates one into such a tile.
 #include <cmath>
 #include <limits>
 
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(NTD, dg_warps_per_sm<R, T>() * 32 / NTD)
 // point q = p + beta (p - p_prev), p_prev read from and p written to the
 // warm-start array (beta = 0: p_prev is not read; write_p = 0: p not written).
 // only_first: the extra step that moves the start of a block with no prox
-// output yet from z to P_B(z) (randomised active sets); chunks of other
+// output yet from z to P_B(z) (randomised active sets); groups of other
 // blocks, and of blocks outside D, leave their scale as it is.
 // Stopping test (inner_tol > 0): p is kept every step; a step k >= 1 also
 // forms the partials ||p - p_prev||^2 and ||p||^2; a block whose test held
@@ -899,9 +900,9 @@ template <int V> struct Count {
 };
 
 // ----------------------------------------------------------------- combine
-// One CTA per active tile (a tile with chunks, or below/right of one):
+// One CTA per active tile (a tile with items, or below/right of one):
 // grid[r][c] = sum of the partial tiles covering the cell, in a fixed order:
-// the cell's own tile's chunks, then the halo rows/columns of the tiles
+// the cell's own tile's items, then the halo rows/columns of the tiles
 // above, left and above-left (periodic grid).  The grid is column-major
 // (element (r, c) at c K0 + r, the layout the inverse column pass reads):
 // the T x T sums, formed from row-major partial-tile reads, are transposed
