@@ -167,31 +167,11 @@ template <typename R> struct VisArgs {
     int *inner_state, *inner_steps;
 };
 
-// Unevaluated sum h + l of two floats, |l| <= ulp(h) / 2: about 48 bits, the
-// accumulator of the FP32 path's norm sums inside a CTA (sums over CTAs are
-// in FP64).  The SM has two FP64 lanes, so a warp's FP64 add holds the pipe
-// for 16 cycles where an FP32 one takes a quarter of a cycle of the SM's
-// issue: the ~10 FP32 instructions of one add below are still 6 times less.
-struct F2 {
-    float h, l;
-};
-__device__ __forceinline__ F2 f2add(F2 a, F2 b) {   // two-sum of the heads, then the tails
-    const float s = a.h + b.h, t = s - a.h;
-    float e = (a.h - (s - t)) + (b.h - t);
-    e += a.l + b.l;
-    const float h = s + e;
-    return isfinite(h) ? F2{h, e - (h - s)} : F2{s, 0.f};
-}
-__device__ __forceinline__ F2 shfl_xor_(F2 v, int m) {
-    return F2{__shfl_xor_sync(0xffffffffu, v.h, m), __shfl_xor_sync(0xffffffffu, v.l, m)};
-}
-__device__ __forceinline__ double shfl_xor_(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
-__device__ __forceinline__ F2 sum_of(F2 a, F2 b) { return f2add(a, b); }
-__device__ __forceinline__ double sum_of(double a, double b) { return a + b; }
-__device__ __forceinline__ double as_double(F2 v) { return (double)v.h + (double)v.l; }
-__device__ __forceinline__ double as_double(double v) { return v; }
-
-// Kahan-compensated FP32 accumulator (FP64 accumulation in the FP64 path).
+// Kahan-compensated FP32 accumulator of one lane (FP64 accumulation in the FP64
+// path).  Only FP64 sums leave it: the sum over the lanes and over runs has
+// FP64's precision and range.  A lane whose sum is big() hands it on before
+// the next group, so that adding another finite square (at most 2^128, and
+// 2^100 is below half its last place) cannot overflow.
 template <typename R> struct Acc {
     R s = 0, c = 0;
     __device__ void add(R x) {
@@ -200,43 +180,37 @@ template <typename R> struct Acc {
         c = (t - s) - y;
         s = t;
     }
-    __device__ auto get() const {   // s - c, unrounded
-        if constexpr (sizeof(R) == 4) {
-            const float h = s - c;
-            return isfinite(h) ? F2{h, (s - h) - c} : F2{s, 0.f};
-        } else {
-            return s - c;
-        }
-    }
+    __device__ double get() const { return (double)s - (double)c; }
+    __device__ bool big() const { return sizeof(R) == 4 && s > R(0x1p100); }
 };
 
-// Warp sums of NV <= 4 values per lane (fixed order).  The first shuffle
+// Warp sums of NV <= 4 values per lane (FP64, fixed order).  The first shuffle
 // steps also halve the number of values a lane carries (lanes whose bit is
 // set take the upper half), so that NV = 2 costs 5 adds a lane instead of
 // 10.  Lane k * warp_sum_step(NV) returns the sum of value k.
 __host__ __device__ constexpr int warp_sum_step(int nv) { return nv <= 1 ? 32 : nv <= 2 ? 16 : 8; }
-template <int NV, typename V> __device__ __forceinline__ V warp_sums(const V (&in)[NV]) {
+template <int NV> __device__ __forceinline__ double warp_sums(const double (&in)[NV]) {
     constexpr int NP = 32 / warp_sum_step(NV);
     const int lane = threadIdx.x & 31;
-    V v[NP];
+    double v[NP];
 #pragma unroll
-    for (int k = 0; k < NP; ++k) v[k] = k < NV ? in[k < NV ? k : 0] : V{};
+    for (int k = 0; k < NP; ++k) v[k] = k < NV ? in[k < NV ? k : 0] : 0.0;
+    auto from = [](double a, int m) { return __shfl_xor_sync(0xffffffffu, a, m); };
     int m = 16;
     if constexpr (NP == 4) {
         const bool hi = lane & m;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) v[k] = sum_of(hi ? v[k + 2] : v[k], shfl_xor_(hi ? v[k] : v[k + 2], m));
+        for (int k = 0; k < 2; ++k) v[k] = (hi ? v[k + 2] : v[k]) + from(hi ? v[k] : v[k + 2], m);
         m >>= 1;
     }
     if constexpr (NP >= 2) {
         const bool hi = lane & m;
-        v[0] = sum_of(hi ? v[1] : v[0], shfl_xor_(hi ? v[0] : v[1], m));
+        v[0] = (hi ? v[1] : v[0]) + from(hi ? v[0] : v[1], m);
         m >>= 1;
     }
-    for (; m > 0; m >>= 1) v[0] = sum_of(v[0], shfl_xor_(v[0], m));
+    for (; m > 0; m >>= 1) v[0] += from(v[0], m);
     return v[0];
 }
-
 
 // a w + c on both components: one instruction on packed pairs in FP32 (the
 // same two roundings as two fmaf), half the issue slots of the taps' sums
@@ -376,6 +350,7 @@ __global__ void __launch_bounds__(NTD, dg_warps_per_sm<R, T>() * 32 / NTD)
         int buf = 0, run = A.warp_run[gw];
         bool fresh = true;    // the group's tile has not been waited for
         bool begin = true;    // the group starts a run
+        bool handed = false;  // the run's slot holds sums of its earlier groups
         bool act = true, first_blk = MODE == DG_FIRST, keep_start = false;
         R mu = 0;
         Acc<R> s_w, s_r;
@@ -458,14 +433,21 @@ __global__ void __launch_bounds__(NTD, dg_warps_per_sm<R, T>() * 32 / NTD)
                     s_r.add(ex * ex + ey * ey);
                 }
             }
-            if (MODE != DG_OP && (!more || Dn.w != D.w)) {   // the run ends
-                const decltype(s_w.get()) part[2] = {s_w.get(), s_r.get()};
-                const auto t = warp_sums<2>(part);
-                if (lane % 16 == 0) A.partials[NPART * (int64_t)A.run_pos[run] + lane / 16] = as_double(t);
-                ++run;
-                s_w = Acc<R>{};
-                s_r = Acc<R>{};
-                begin = true;
+            if (MODE != DG_OP) {
+                const bool end = !more || Dn.w != D.w;   // the run ends
+                if (end || __any_sync(0xffffffffu, s_w.big() || s_r.big())) {
+                    const double part[2] = {s_w.get(), s_r.get()};
+                    const double t = warp_sums<2>(part);
+                    if (lane % 16 == 0) {
+                        double *slot = A.partials + NPART * (int64_t)A.run_pos[run] + lane / 16;
+                        *slot = handed ? *slot + t : t;
+                    }
+                    s_w = Acc<R>{};
+                    s_r = Acc<R>{};
+                    run += end;
+                    begin = end;
+                    handed = !end;
+                }
             }
             if (next_tile) {
                 __syncwarp();   // every lane has read the tile: its buffer may be refilled
@@ -525,7 +507,7 @@ __global__ void __launch_bounds__(SUB_NT) k_subiter(VisArgs<R> A, int only_first
         int4 D = A.grp[g0];
         In cur;
         if (lane < D.y) load(D.x + lane, cur);
-        bool begin = true, skip = false;
+        bool begin = true, skip = false, handed = false;   // handed: as in the degridding
         R c = 0, mu = 0;
         Acc<R> s_w, s_d, s_n;
         for (int g = g0; g < g1; ++g) {
@@ -560,17 +542,27 @@ __global__ void __launch_bounds__(SUB_NT) k_subiter(VisArgs<R> A, int only_first
                 const R dx = wn.x - yy.x, dy = wn.y - yy.y;
                 s_w.add(dx * dx + dy * dy);
             }
-            if (!more || Dn.w != D.w) {   // the run ends
+            const bool end = !more || Dn.w != D.w;   // the run ends
+            if (end || __any_sync(0xffffffffu, s_w.big() || s_d.big() || s_n.big())) {
                 if (!skip) {
-                    const decltype(s_w.get()) part[3] = {s_w.get(), s_d.get(), s_n.get()};
-                    const auto t = warp_sums<3>(part);
-                    // slot 1 keeps the degridding's residual
-                    if (lane % 8 == 0 && lane < 24)
-                        A.partials[NPART * (int64_t)A.run_pos[run] + (lane ? lane / 8 + 1 : 0)] = as_double(t);
+                    double *slot = A.partials + NPART * (int64_t)A.run_pos[run];
+                    // (a warp's FP64 add holds the pipe of the SM's two lanes for 16
+                    // cycles: only the sums that are read are formed)
+                    if (test_out) {
+                        const double part[3] = {s_w.get(), s_d.get(), s_n.get()};
+                        const double t = warp_sums<3>(part);
+                        // slot 1 keeps the degridding's residual
+                        slot += lane ? lane / 8 + 1 : 0;
+                        if (lane % 8 == 0 && lane < 24) *slot = handed ? *slot + t : t;
+                    } else {
+                        const double part[1] = {s_w.get()}, t = warp_sums<1>(part);
+                        if (lane == 0) *slot = handed ? *slot + t : t;
+                    }
                 }
-                ++run;
                 s_w = s_d = s_n = Acc<R>{};
-                begin = true;
+                run += end;
+                begin = end;
+                handed = !end;
             }
             D = Dn;
             cur = nx;
