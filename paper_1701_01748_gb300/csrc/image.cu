@@ -3,6 +3,8 @@
 // arguments of the primal step of Algorithm 3 (projection onto the positive
 // orthant, Section 3.3 Eq. "proj-plus"), whose kernel is fused with the row
 // FFT passes in fft.cu.
+#include <cmath>
+
 #include "common.cuh"
 
 namespace ppd {
@@ -111,9 +113,11 @@ template <typename R> PrimalArgs<R> primal_args(ppd_ctx *c) {
     P.ut = static_cast<const R *>(c->ut);
     P.w0 = static_cast<const R *>(c->wgt);
     P.xtrue = static_cast<const R *>(c->xtrue);
-    P.tau = (R)c->tau;
-    P.eta = (R)c->eta;
-    P.zeta = (R)(c->zeta / c->psiw2);
+    const double step = c->tau * c->eta;
+    P.step_g = (R)step;
+    if ((double)P.step_g >= step) P.step_g = std::nextafter(P.step_g, R(0));
+    P.step_gl = (R)(step - (double)P.step_g);
+    P.step_u = (R)(c->tau * (c->zeta / c->psiw2));
     P.kappa = (R)(c->kappa * c->psiw2);
     P.pmask = c->rand_on ? c->mask_cur + c->d : nullptr;
     return P;

@@ -83,8 +83,12 @@ __global__ void k_cell_count(const int32_t *__restrict__ cell, const int32_t *__
 // chains).  The coefficients p[j KB_N + k] of t^k are kernel arguments, so
 // with the loops unrolled each is a constant-bank operand: no load.
 //
-// FP32: 8 coefficients, fit error 4e-8, below the rounding (8.6e-8 at most,
-// 2.2e-8 rms against 64-bit values; Horner had 8.2e-8, 2.1e-8).
+// FP32: 8 coefficients, fit error 4e-8 at most, 1.5e-8 rms.  The constant
+// term of the two inner taps (weights up to 1) keeps the part that rounding
+// it to FP32 drops (kbl), and is added last: every visibility sees the same
+// coefficients, so without it the whole operator's amplitude was 4e-8 low
+// (and the weights 2.2e-8 rms off, where eight Horner chains had 2.0e-8; with
+// it 1.85e-8, 9.5e-8 at most).  It costs 8 adds a visibility.
 // FP64: 16 coefficients reach 2.2e-16 at most, 4e-17 rms for the default
 // shape beta = 2.34 J, closer than the Bessel function itself, whose 16
 // evaluations a visibility were most of the FP64 visibility kernels' time on
@@ -107,14 +111,19 @@ template <typename R, typename A> __device__ __forceinline__ void kb_weights(R f
     const R t = fma(R(2), frac, R(-1)), s = t * t;
 #pragma unroll
     for (int j = 0; j < KB_J / 2; ++j) {
+        const bool split = sizeof(R) == 4 && j >= KB_J / 4;   // constant term in two parts
         R e = args.kbp[j * N + N - 2], o = args.kbp[j * N + N - 1];
 #pragma unroll
         for (int k = N - 4; k >= 0; k -= 2) {
-            e = fma(e, s, args.kbp[j * N + k]);
+            e = fma(e, s, split && k == 0 ? args.kbl[j - KB_J / 4] : args.kbp[j * N + k]);
             o = fma(o, s, args.kbp[j * N + k + 1]);
         }
         w[j] = fma(o, t, e);
         w[KB_J - 1 - j] = fma(-o, t, e);
+        if (split) {
+            w[j] += args.kbp[j * N];
+            w[KB_J - 1 - j] += args.kbp[j * N];
+        }
     }
 }
 
@@ -137,6 +146,7 @@ template <typename R> struct VisArgs {
     int n_warps;
     int K0, K1, ntile1;
     R kbp[KB_J / 2 * KB_N<R>];   // the weight polynomials (kb_weights)
+    R kbl[KB_J / 4];             // FP32: what rounding dropped of the inner taps' constant terms
     int bessel;                  // FP64: the weights come from the Bessel function
     double beta, inv_i0b;
     const cplx_t<R> *y;
@@ -977,6 +987,10 @@ template <typename R> VisArgs<R> make_args(ppd_ctx *c) {
     A.K1 = c->K1;
     A.ntile1 = c->K1 / c->T;
     for (int i = 0; i < KB_J / 2 * KB_N<R>; ++i) A.kbp[i] = (R)c->kbpoly_h[i];
+    for (int i = 0; i < KB_J / 4; ++i) {
+        const int at = (KB_J / 4 + i) * KB_N<R>;
+        A.kbl[i] = (R)(c->kbpoly_h[at] - (double)A.kbp[at]);
+    }
     A.bessel = c->kb_bessel;
     A.beta = c->beta;
     A.inv_i0b = c->kb_inv_i0b;
