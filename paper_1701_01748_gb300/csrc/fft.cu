@@ -556,6 +556,25 @@ __device__ __forceinline__ void load_two_real_any(const cplx_t<R> *__restrict__ 
         }
     }
 }
+// The spectra of rows row0 + s, s < nseq, one to a sequence, conjugated and in
+// natural order, so that the real parts of the forward FFT are those of the
+// inverse.  The operator's inverse rows go this way: a row's own transform has
+// half of its rounding in the imaginary part, which is dropped, where a pair's
+// has the other row there (adjoint at 960 x 400, error against 64 bits: 1.55e-7
+// in pairs, 1.32e-7 by single rows; 78 and 81 us).  The iteration's fused pass
+// keeps pairs: its images are as close either way (1.08e-7 at 160^2, 1.04e-7 at
+// 240^2) and 144 x 80 takes 61 us an iteration against 65.
+template <typename R>
+__device__ __forceinline__ void load_rows_inverse(const cplx_t<R> *__restrict__ tmp, int row0, int L0, int K, int nseq,
+                                                  cplx_t<R> *buf) {
+    for (int s = 0; s < nseq; ++s) {
+        const int r = row0 + s;
+#pragma unroll 4
+        for (int c = threadIdx.x; c < K; c += NTR)   // column c holds frequency (c + K/2) mod K
+            buf[mplace<false>(s, wrapK(c + K / 2, K), K, 0)] =
+                r < L0 ? cconj(tmp[(int64_t)r * K + c]) : cplx_t<R>{0, 0};
+    }
+}
 template <typename R>
 __device__ __forceinline__ void store_two_real_any(const cplx_t<R> *out, int row0, int L0, int K, int nseq,
                                                    const uint8_t *__restrict__ colmask, cplx_t<R> *__restrict__ tmp) {
@@ -752,19 +771,16 @@ __global__ void __launch_bounds__(row_nt<R, KT>(), pass_ctas<R, KT>()) k_rows_in
             });
         return;
     }
-    const int K = pa.pl.K, B = pa.nseq, row0 = blockIdx.x * 2 * B;
+    const int K = pa.pl.K, B = pa.nseq, row0 = blockIdx.x * B;
     C *buf2 = buf + B * mpad(K);
-    load_two_real_any<R>(tmp, row0, L0, K, B, buf);
+    load_rows_inverse<R>(tmp, row0, L0, K, B, buf);
     __syncthreads();
     const C *out = fft_any<R, NTR, false>(buf, buf2, B, 0, pa.pl, tw);
-    for (int s = 0; s < B; ++s) {
-        const int ra = row0 + 2 * s, rb = ra + 1;
-        const R fa = ra < L0 ? s0[ra] : R(0), fb = rb < L0 ? s0[rb] : R(0);
-        for (int n1 = threadIdx.x; n1 < L1; n1 += NTR) {
-            const C v = out[mplace<false>(s, wrapK(n1 - L1 / 2 + K, K), K, 0)];
-            if (ra < L0) img[(int64_t)ra * L1 + n1] = fa * s1[n1] * v.x;
-            if (rb < L0) img[(int64_t)rb * L1 + n1] = -fb * s1[n1] * v.y;
-        }
+    for (int s = 0; s < B && row0 + s < L0; ++s) {
+        const R f = s0[row0 + s];
+        for (int n1 = threadIdx.x; n1 < L1; n1 += NTR)
+            img[(int64_t)(row0 + s) * L1 + n1] =
+                f * s1[n1] * out[mplace<false>(s, wrapK(n1 - L1 / 2 + K, K), K, 0)].x;
     }
 }
 
@@ -911,7 +927,9 @@ template <typename R, int KT> struct RowPass {
         PPD_CHECK(smem_attr((const void *)k_rows_inv<R, KT>, sh));
         int site;
         PPD_CHECK(launch_begin(c, "fft_inv_rows", s, &site));
-        launch(c, true, k_rows_inv<R, KT>, blocks(c), NTH, sh, s, static_cast<const cplx_t<R> *>(c->fft_tmp_inv),
+        // (the mixed-radix core inverts single rows)
+        const unsigned n = KT ? blocks(c) : (unsigned)((c->L0 + nseq(c) - 1) / nseq(c));
+        launch(c, true, k_rows_inv<R, KT>, n, NTH, sh, s, static_cast<const cplx_t<R> *>(c->fft_tmp_inv),
                img, tw(c), static_cast<const R *>(c->deap0), static_cast<const R *>(c->deap1), c->L0, c->L1,
                args(c));
         return launch_end(c, site, s);
