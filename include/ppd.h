@@ -364,7 +364,8 @@ PPD_API int ppd_op_adjoint_noalloc(ppd_ctx *ctx, const void *y_dev, void *x_dev,
 
 /* Psi^dagger x (Section 2.2, Section 5.1: Dirac + db1..db8, 4 levels,
  * periodic, Mallat layout, each basis scaled by 1/3): x_dev n0*n1 reals ->
- * c_dev 9*n0*n1 reals (basis-major).  Enqueued on stream. */
+ * c_dev 9*n0*n1 reals (basis-major).  x_dev may be c_dev, the image then
+ * lying in the Dirac part that the call replaces.  Enqueued on stream. */
 PPD_API int ppd_psi_analysis(ppd_ctx *ctx, const void *x_dev, void *c_dev, void *stream);
 
 /* Psi c = (1/3) sum_i Psi_i c_i: c_dev 9*n0*n1 reals -> x_dev n0*n1 reals. */

@@ -283,7 +283,8 @@ __device__ __forceinline__ void ana_tile(const R *__restrict__ src, int in_pitch
 //         (MODE 0: c = D x / 3) or clip-updated (1: u = clip(u + D x / 3, kappa);
 //         2: u = clip(u + w D x / 3, kappa), w the prior weights wgt, laid out
 //         like coef)
-//   dirac: MODE 0, level 0: the Dirac basis's coefficients x / 3, or null
+//   dirac: MODE 0, level 0: the Dirac basis's coefficients x / 3, or null (in
+//         must not overlap them)
 //   pmask: active set P of Algorithm 3 (9 flags, Dirac first) or null; in
 //         modes 1 and 2 a basis outside P keeps u_b and is skipped at every level
 template <typename R, int TS, int MODE>
@@ -608,7 +609,7 @@ template <typename R> int analysis_all(ppd_ctx *c, const R *x, R *coef, int mode
             PPD_CHECK(launch_begin(c, "sara_analysis", s, &site));
             launch(c, l > 0, k, dim3(tiles(n0 / 2, n1 / 2, TS), N_WAVELETS), NT, ana_smem<R, TS>(), s, in, pitch,
                    bstride, n0, n1, ll[l & 1], ll_stride, (int)last, coef, wgt, L1, N, alpha,
-                   mode == 0 && l == 0 ? coef : nullptr, pmask);
+                   mode == 0 && l == 0 && x != coef ? coef : nullptr, pmask);
             return launch_end(c, site, s);
         };
         PPD_CHECK(large_tile<R>(tiles(n0 / 2, n1 / 2, 32) * N_WAVELETS) ? go(Int<32>{}) : go(Int<16>{}));
@@ -759,7 +760,9 @@ int make_filters(ppd_ctx *c) {
 }
 
 template <typename R> int psi_analysis(ppd_ctx *c, const R *x, R *coef, cudaStream_t s) {
-    return analysis_all<R>(c, x, coef, 0, s);
+    PPD_CHECK(analysis_all<R>(c, x, coef, 0, s));
+    // an image that lies in the Dirac part itself is scaled once every basis has read it
+    return x == coef ? scale_copy<R>(c, x, coef, c->N, 1.0 / 3.0, s) : PPD_OK;
 }
 
 template <typename R> int psi_synthesis(ppd_ctx *c, const R *coef, R *x, cudaStream_t s) {
