@@ -771,7 +771,7 @@ def main():
                    "l2": "flushed (256 MiB write) between timed steps", "graph": "one CUDA graph per iteration",
                    "replicas": world,
                    "launches": "overlapped (programmatic dependent launch)" if args.launch_overlap else "serial",
-                   "gridding": {"tile": prm32["tile"], "chunk": prm32["chunk"], "work_items": prm32["n_chunks"],
+                   "gridding": {"tile": prm32["tile"], "chunk": prm32["chunk"], "tile_block_runs": prm32["n_chunks"],
                                 "grid_warps": prm32["grid_warps"], "degrid_threads": prm32["degrid_threads"],
                                 "autotuned": not args.no_autotune and args.tile == 0 and args.chunk == 0}},
         "snr_iters": snr_iters,

@@ -709,8 +709,10 @@ int ppd_create(ppd_ctx **out, const ppd_config *cfg) {
     c->zeta = k.zeta > 0 ? k.zeta : 1.0;
     cudaGetDevice(&c->device);
     {
-        int major = 0;
+        int major = 0, sms = 0;
         cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+        c->sms = std::max(sms, 1);
         c->overlap = k.launch_overlap == 1 && major >= 9;
     }
     auto bail = [&](int st) {
@@ -957,9 +959,7 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     // 1024^2: 11.05 ms with one piece, 10.96 with up to four; every piece
     // ends a run, and eight made the degridding 11 % longer in instructions)
     const int64_t ng = (int64_t)grp.size();
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    const int64_t nwarps = std::min<int64_t>(ng, (int64_t)std::max(sms, 1) * degrid_warps_per_sm(c));
+    const int64_t nwarps = std::min<int64_t>(ng, (int64_t)c->sms * degrid_warps_per_sm(c));
     const int64_t rounds = std::max<int64_t>(1, std::min<int64_t>(4, ng / (4 * nwarps)));
     std::vector<int32_t> wgrp(nwarps + 1, 0), wrun(nwarps + 1, 0), rblk;
     {
@@ -994,7 +994,7 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     std::vector<int32_t> cord(nch);
     for (int64_t k = 0; k < nch; ++k) cord[k] = (int32_t)k;
     std::stable_sort(cord.begin(), cord.end(), [&](int32_t a, int32_t b) { return it[a].y > it[b].y; });
-    const int small = ng >= 64LL * std::max(sms, 1) ? 4 : 1;
+    const int small = ng >= 64LL * c->sms ? 4 : 1;
     int64_t n_large = 0;
     while (n_large < nch && it[cord[n_large]].y > small) ++n_large;
     c->ch.n = nch;
@@ -1007,7 +1007,7 @@ int ppd_set_visibilities(ppd_ctx *c, int64_t M, const double *uv, const double *
     // warps while the items make few waves, four (more CTAs per SM) beyond
     // twelve items per SM
     if (c->cfg.grid_warps == 0 && !c->shape_tuned && c->is_f32) {
-        c->grid_nw = nch > 12LL * std::max(sms, 1) ? 4 : 8;
+        c->grid_nw = nch > 12LL * c->sms ? 4 : 8;
     }
     c->ch.n_active = (int64_t)active.size();
     const size_t cbsz = 2 * c->rsz;

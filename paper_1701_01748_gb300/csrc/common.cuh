@@ -181,7 +181,7 @@ struct ppd_ctx {
     double beta = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    int device = 0;
+    int device = 0, sms = 1;   // the device and its SMs
 
     // image side
     void *x = nullptr, *xt = nullptr, *g = nullptr, *ut = nullptr, *xtrue = nullptr;

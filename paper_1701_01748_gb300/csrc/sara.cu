@@ -580,9 +580,15 @@ inline unsigned tiles(int h0, int h1, int ts) { return (unsigned)(((h0 + ts - 1)
 template <int V> struct Int {
     static constexpr int value = V;
 };
-// Large tiles once they give every SM two CTAs (FP64 keeps the small ones:
-// its two FP64 lanes per SM, not the halo, bound it).
-template <typename R> bool large_tile(unsigned ctas) { return sizeof(R) == 4 && ctas >= 304; }
+// go(tile side) for a level with quadrants of h0 x h1: large tiles once they
+// give every SM two CTAs of the eight bases (FP64 keeps the small ones: its
+// two FP64 lanes per SM, not the halo, bound it).
+template <typename R, typename Go> int with_tile(const ppd_ctx *c, int h0, int h1, Go go) {
+    if constexpr (sizeof(R) == 4) {
+        if (tiles(h0, h1, 32) * N_WAVELETS >= 2u * c->sms) return go(Int<32>{});
+    }
+    return go(Int<16>{});
+}
 
 // Analysis of all levels (tiled).  mode 0 writes c = D x / 3, mode 1
 // clip-updates u with the prior weights and the clip level kappa ||Psi W||^2.
@@ -612,7 +618,7 @@ template <typename R> int analysis_all(ppd_ctx *c, const R *x, R *coef, int mode
                    mode == 0 && l == 0 && x != coef ? coef : nullptr, pmask);
             return launch_end(c, site, s);
         };
-        PPD_CHECK(large_tile<R>(tiles(n0 / 2, n1 / 2, 32) * N_WAVELETS) ? go(Int<32>{}) : go(Int<16>{}));
+        PPD_CHECK(with_tile<R>(c, n0 / 2, n1 / 2, go));
     }
     return PPD_OK;
 }
@@ -638,7 +644,7 @@ int synthesis_levels(ppd_ctx *c, const R *coef, const R *wgt, const R **ll0, cud
                    coef, wgt, L1, N, coarsest ? coef : prev, coarsest ? 1 : 0, st, n0, n1, buf[k & 1], st);
             return launch_end(c, site, s);
         };
-        PPD_CHECK(large_tile<R>(tiles(n0 / 2, n1 / 2, 32) * N_WAVELETS) ? go(Int<32>{}) : go(Int<16>{}));
+        PPD_CHECK(with_tile<R>(c, n0 / 2, n1 / 2, go));
         prev = buf[k & 1];
     }
     *ll0 = prev;
@@ -660,7 +666,7 @@ int synthesis_final(ppd_ctx *c, const R *coef, const R *wgt, const R *ll0, const
                L0, L1, c->N, from_coef ? coef : ll0, from_coef ? 1 : 0, st, dirac, scale, out);
         return launch_end(c, site, s);
     };
-    return large_tile<R>(tiles(L0 / 2, L1 / 2, 32) * N_WAVELETS) ? go(Int<32>{}) : go(Int<16>{});
+    return with_tile<R>(c, L0 / 2, L1 / 2, go);
 }
 
 // Durand-Kerner roots of the polynomial with real coefficients a (ascending).

@@ -27,7 +27,6 @@ namespace ppd {
 namespace {
 
 template <typename C> __device__ __forceinline__ C cadd(C a, C b) { return C{a.x + b.x, a.y + b.y}; }
-template <typename C> __device__ __forceinline__ C csub(C a, C b) { return C{a.x - b.x, a.y - b.y}; }
 
 // ----------------------------------------------------------------- binning
 // kappa = (omega * K) * (1/(2 pi)) with correctly rounded multiplies (no FMA
@@ -154,10 +153,8 @@ template <typename R> struct VisArgs {
     const R *mu;
     const R *scale;              // per block: the P_B scale of the last step (k_block_scale)
     double *partials;            // norm partials of the runs
-    // partials live in block-major slots: run r writes slot run_pos[r];
-    // block b's slots are blk_ptr[b] .. blk_ptr[b+1] - 1
-    const int32_t *blk_ptr, *run_pos;
-    const double *eps;
+    // partials live in block-major slots: run r writes slot run_pos[r]
+    const int32_t *run_pos;
     int *err;
     // randomised active sets (null: every block active): the current
     // iteration's block flags, per-block "has a prox output" flags, and the
@@ -1008,13 +1005,11 @@ template <typename R> VisArgs<R> make_args(ppd_ctx *c) {
     A.mu = static_cast<const R *>(c->mu_d);
     A.scale = static_cast<const R *>(c->scale);
     A.partials = c->partials;
-    A.blk_ptr = c->ch.blk_ptr;
     A.run_pos = c->ch.run_pos;
     A.warp_run = c->ch.warp_run;
     A.grp = c->ch.grp;
     A.warp_grp = c->ch.warp_grp;
     A.n_warps = c->ch.n_warps;
-    A.eps = c->eps_d;
     A.err = c->err;
     A.bmask = c->rand_on ? c->mask_cur : nullptr;
     A.seen = c->rand_on ? c->blk_seen : nullptr;
