@@ -62,7 +62,7 @@ extern "C" {
 
 /* precision (config.precision) */
 #define PPD_FP64_PLAIN          0   /* every array and reduction in double, kernels launched one by one */
-#define PPD_FP32_FP64NORMS      1   /* float arrays, double norms / bounds / stop tests, one CUDA graph per iteration */
+#define PPD_FP32_FP64NORMS      1   /* float arrays, double norms (of squares formed in float) / bounds / stop tests, one CUDA graph per iteration */
 
 /* Algorithm 2 start point (config.inner_init) */
 #define PPD_INNER_WARM          0   /* previous iteration's prox output (P_B(z) on the first iteration) */
@@ -137,7 +137,8 @@ typedef struct {
     int32_t  pad1;
 } ppd_config;
 
-/* Per-call statistics (ppd_iterate).  All norms are computed in double. */
+/* Per-call statistics (ppd_iterate).  All norms are computed in double, in the
+ * float precision from squares formed in float. */
 typedef struct {
     int32_t  iters_done;        /* PPD iterations completed by this context so far */
     int32_t  status;            /* status of the call */

@@ -6,9 +6,9 @@
 //                      column pass tmp              -> grid (K0 x K1 complex)
 // Inverse  Re(Z^T F^H grid): column pass grid -> tmp, row pass tmp -> image.
 //
-// Every pass is a batched Stockham FFT: a CTA takes B whole rows (row pass,
-// length K1) or a strip of W columns (column pass, length K0), runs the
-// stages and writes the result.  Only the L nonzero rows / columns of the
+// Every pass is a batched Stockham FFT: a CTA takes B sequences of one or two
+// whole rows (row pass, length K1) or a strip of W columns (column pass, length
+// K0), runs the stages and writes the result.  Only the L nonzero rows / columns of the
 // padded image are read or produced; the grid is stored with the zero
 // frequency at the centre (plain index k at (k + K/2) mod K).
 //
@@ -133,9 +133,10 @@ template <typename R, int N> __device__ __forceinline__ void dft_regs(cplx_t<R> 
 // t + b TPS take inputs j + q K/RAD, twiddled by w^(q k K/(Ns RAD)), k = j mod
 // Ns, and give outputs (j - k) RAD + k + p Ns.  Inputs and outputs of the
 // whole transform that thread t sees are the positions t + m TPS, m < EPT.
-// Passes are few (three from K = 512 on) because each crosses shared memory:
-// a radix-4 core went through it seven times at K = 8192 with up to 4-way
-// bank conflicts and was bound by it (75 % of the data path busy).  PAD adds
+// Passes are few (two to four, the last of the radix that is left: 8 8 at K =
+// 64, 8 8 8 2 for FP32 rows of 1024, 16 16 32 at 8192) because each crosses
+// shared memory: a radix-4 core went through it seven times at K = 8192 with up
+// to 4-way bank conflicts and was bound by it (75 % of the data path busy).  PAD adds
 // one element per 16, so that the stride-RAD stores of the first pass fall
 // in distinct banks.
 template <typename R_, int K_, int EPT_> struct Fft {
@@ -462,8 +463,8 @@ struct PassArgs {
     int nseq, lseq;   // lseq: log2 of nseq (columns)
 };
 
-// Row passes of the power-of-two core transform two real rows (a, b) as one
-// complex sequence.  Forward: z = a + i b, and after the FFT
+// Row passes transform two real rows (a, b) as one complex sequence (but for
+// the mixed-radix core's k_rows_inv: load_rows_inverse).  Forward: z = a + i b, and after the FFT
 // A[k] = (Z[k] + conj(Z[-k]))/2, B[k] = (Z[k] - conj(Z[-k]))/(2i).
 template <typename C> __device__ __forceinline__ void split_two_real(C z, C zr, C &A, C &B) {
     using R = decltype(z.x);

@@ -112,9 +112,10 @@ template <typename R> constexpr int piece(int n) { return n * (int)sizeof(R) >= 
 // and the issue slots full.  TS = 32 reads 1.5 times its input (halo), TS =
 // 16 2.1 times; the small tile serves levels that would not give every SM
 // two large ones, and FP64.  Level 0 before -> now: analysis 118 -> 61 us at
-// 2048^2, 38 -> 26 us at 1024^2, 12.7 -> 8.9 us at 512^2; synthesis 176 -> 100,
-// 47 -> 28, 15.5 -> 10.1 us.  Issue slots bound the analysis (81 % busy at
-// 2048^2, FMAs under half of them).  Row pitches are 4 mod 8 floats with 8 rows in
+// 2048^2 (67 with the Dirac basis, which had a launch of 9), 38 -> 26 us at
+// 1024^2, 12.7 -> 9.3 us at 512^2; synthesis 176 -> 100, 47 -> 28, 15.5 -> 10.1
+// us.  Issue slots bound the analysis (80 % busy at 2048^2, FMAs under half of
+// them).  Row pitches are 4 mod 8 floats with 8 rows in
 // distinct banks for 16-byte accesses of lanes in consecutive rows.
 template <int TS> struct AnaGeo {
     static constexpr int EXT = 2 * TS + MAX_TAPS - 2;           // input tile side (78 / 46)

@@ -289,12 +289,12 @@ template <int E> __device__ __forceinline__ double2 footprint(const double2 *cel
 // barrier separates the groups: with a CTA per work item (a tile's
 // visibilities of one block) and its barriers, warps waited at barriers for
 // 5 of every 14 cycles per issued instruction and small items left most
-// lanes idle.  Before -> now, with the dual step: 28.4 -> 16.8 us at 512^2
-// (524k visibilities), 159 -> 98 us at 1024^2 (4.2M), 42 -> 22 us at 640 x 480
-// (700k); without it 522 -> 237 us at 4096^2 (8.4M).  What bounds it now is
+// lanes idle.  Before -> now, with the dual step: 28.4 -> 17.9 us at 512^2
+// (524k visibilities), 159 -> 97 us at 1024^2 (4.2M), 42 -> 23 us at 640 x 480
+// (700k); without it 522 -> 223 us at 4096^2 (8.4M).  What bounds it now is
 // the shared-memory reads (64 eight-byte reads a visibility, two passes each
-// for a warp: 52 us of the SM's data path at 1024^2) and the issue slots
-// (61 % busy there).
+// for a warp: 51 % of the SM's data path at 1024^2, 70 % at 4096^2 without the
+// dual step) and the issue slots (61 and 46 % busy).
 template <typename R> struct VisIn {
     VisRec<R> rc;
     cplx_t<R> v, y, p;
@@ -314,11 +314,16 @@ __device__ __forceinline__ void load_vis(const VisArgs<R> &A, int gi, VisIn<R> &
 
 // Warps per SM the degridding's shared memory and registers allow, and with
 // them the shares of the groups (a share per resident warp).  T = 32: one
-// tile buffer a warp (the copy is then waited for).
+// tile buffer a warp (the copy is then waited for, with four times the
+// visibilities behind each): 125 us with CTA work items and two buffers, 89 with
+// one a warp at 1024^2; 27 and 22 at 512^2.
 template <typename R, int T> constexpr int dg_warps_per_sm() { return sizeof(R) == 8 ? 8 : T == 16 ? 24 : 16; }
 template <int T> constexpr int dg_bufs() { return T == 16 ? 2 : 1; }
 
-// NTD threads per CTA (256 or 128; FP64: 256): the CTA only groups warps.
+// NTD threads per CTA (256 or 128; FP64: 256): the CTA only groups warps.  Which
+// is faster follows no rule: an iteration takes 322 us with 256 and 324 with 128
+// at 1024^2, 91.1 and 91.0 at 512^2, 60.8 and 62.4 at 256^2, 46.3 and 44.8 at
+// 128^2 (8 gridding warps, 4 at 1024^2), and on other coverages the other way.
 template <typename R, int T, int MODE, int NTD>
 __global__ void __launch_bounds__(NTD, dg_warps_per_sm<R, T>() * 32 / NTD)
     k_degrid(const __grid_constant__ CUtensorMap tmap, int use_tma, const cplx_t<R> *__restrict__ grid, VisArgs<R> A,
@@ -686,11 +691,11 @@ __global__ void k_block_norms(const double *__restrict__ partials, const int32_t
 // item of one block and a CTA per item left most warps idle (4096^2, 8.4M
 // visibilities in 256 blocks: 81k items of 103 on average, 5700
 // instructions each, against 36k of 2 to 32 groups now).  Before -> now: 644 ->
-// 359 us there (and the combine pass, with half the partial tiles, 138 ->
-// 112), 125 -> 111 us at 1024^2 (4.2M visibilities, 64 blocks, dual step), 37
-// -> 29 us at 640 x 480 (700k), 27 -> 28 us at 512^2 (524k).  What bounds it
-// now: issue slots (71 % busy at 1024^2, 20 instructions a visibility) and
-// the shared-memory path (71 %).
+// 361 us there (and the combine pass, with half the partial tiles, 138 ->
+// 112), 125 -> 107 us at 1024^2 (4.2M visibilities, 64 blocks, dual step), 37
+// -> 29 us at 640 x 480 (700k), 27 -> 29 us at 512^2 (524k).  What bounds it
+// now: issue slots (73 % busy at 1024^2, 22 instructions a visibility) and
+// the shared-memory path (63 %).
 // With the private-tile pitch T + 8 = 8 mod 16 (in 8-byte words) rows a and a
 // + 2 share banks: lanes of rows 2, 3, 6 and 7 take column b + 4 first.
 // A warp's staging area: per visibility w0[a] Theta v and the pairs (w1[b],
