@@ -398,9 +398,9 @@ __device__ __forceinline__ void syn_compute(const R *q, R *tl, R *th, R (&acc)[N
     for (int task = threadIdx.x; task < 2 * EXT * NR; task += NT) {
         const int half = task >= EXT * NR, s = task - half * EXT * NR, j = s % EXT, p0 = (s / EXT) * PS;
         const R *qa = q + (half * G::EXT + p0) * G::PQ + 9 - H + j, *qb = qa + 2 * G::EXT * G::PQ;
-        R e[PS], o[PS];
+        R e[PS], o[PS], eh[PS], oh[PS];   // low and high half apart: fewer roundings at the sum's size
 #pragma unroll
-        for (int p = 0; p < PS; ++p) e[p] = o[p] = R(0);
+        for (int p = 0; p < PS; ++p) e[p] = o[p] = eh[p] = oh[p] = R(0);
 #pragma unroll
         for (int i = 0; i < PS + H - 1; ++i) {   // tile row p0 + i serves tap pair kk = p + H - 1 - i
             const R a = qa[i * G::PQ], d = qb[i * G::PQ];
@@ -410,16 +410,16 @@ __device__ __forceinline__ void syn_compute(const R *q, R *tl, R *th, R (&acc)[N
                 if (kk >= 0 && kk < H) {
                     e[p] = fma(f.h(2 * kk), a, e[p]);
                     o[p] = fma(f.h(2 * kk + 1), a, o[p]);
-                    e[p] = fma(f.g(2 * kk), d, e[p]);
-                    o[p] = fma(f.g(2 * kk + 1), d, o[p]);
+                    eh[p] = fma(f.g(2 * kk), d, eh[p]);
+                    oh[p] = fma(f.g(2 * kk + 1), d, oh[p]);
                 }
             }
         }
         R *dst = (half ? th : tl) + 2 * p0 * G::PT + j;
 #pragma unroll
         for (int p = 0; p < PS; ++p) {
-            dst[2 * p * G::PT] = e[p];
-            dst[(2 * p + 1) * G::PT] = o[p];
+            dst[2 * p * G::PT] = e[p] + eh[p];
+            dst[(2 * p + 1) * G::PT] = o[p] + oh[p];
         }
     }
     __syncthreads();
@@ -430,6 +430,7 @@ __device__ __forceinline__ void syn_compute(const R *q, R *tl, R *th, R (&acc)[N
         R a[PS + H - 1], d[PS + H - 1];
         load_row<piece<R>(PS)>(tl + m * G::PT + p0, a);
         load_row<piece<R>(PS)>(th + m * G::PT + p0, d);
+        R high[2 * PS] = {};
 #pragma unroll
         for (int i = 0; i < PS + H - 1; ++i)
 #pragma unroll
@@ -438,10 +439,12 @@ __device__ __forceinline__ void syn_compute(const R *q, R *tl, R *th, R (&acc)[N
                 if (kk >= 0 && kk < H) {
                     acc[t][2 * p] = fma(f.h(2 * kk), a[i], acc[t][2 * p]);
                     acc[t][2 * p + 1] = fma(f.h(2 * kk + 1), a[i], acc[t][2 * p + 1]);
-                    acc[t][2 * p] = fma(f.g(2 * kk), d[i], acc[t][2 * p]);
-                    acc[t][2 * p + 1] = fma(f.g(2 * kk + 1), d[i], acc[t][2 * p + 1]);
+                    high[2 * p] = fma(f.g(2 * kk), d[i], high[2 * p]);
+                    high[2 * p + 1] = fma(f.g(2 * kk + 1), d[i], high[2 * p + 1]);
                 }
             }
+#pragma unroll
+        for (int k = 0; k < 2 * PS; ++k) acc[t][k] += high[k];
     }
 }
 
