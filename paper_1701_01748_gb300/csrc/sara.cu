@@ -113,7 +113,7 @@ template <typename R> constexpr int piece(int n) { return n * (int)sizeof(R) >= 
 // 16 2.1 times; the small tile serves levels that would not give every SM
 // two large ones, and FP64.  Level 0 before -> now: analysis 118 -> 61 us at
 // 2048^2 (67 with the Dirac basis, which had a launch of 9), 38 -> 26 us at
-// 1024^2, 12.7 -> 9.3 us at 512^2; synthesis 176 -> 100, 47 -> 28, 15.5 -> 10.1
+// 1024^2, 12.7 -> 9.6 us at 512^2; synthesis 176 -> 101, 47 -> 28, 15.5 -> 10.5
 // us.  Issue slots bound the analysis (80 % busy at 2048^2, FMAs under half of
 // them).  Row pitches are 4 mod 8 floats with 8 rows in
 // distinct banks for 16-byte accesses of lanes in consecutive rows.
@@ -385,6 +385,10 @@ __device__ __forceinline__ void syn_load(R *q, const R *__restrict__ cb, const R
     copy_commit();
 }
 
+// The low and the high half of a pass are summed apart: in one accumulator every
+// addition rounds at the size of the whole sum (error of Psi against 64 bits
+// 1.24e-7 of the image, apart 1.18e-7; level 0 at 2048^2 100 and 101 us).
+//
 // The two filter passes over complete quadrant tiles (a barrier behind them);
 // adds the outputs of this thread's tasks to acc: task t = row task % 2TS,
 // samples 2 PS (task / 2TS) .. + 2 PS - 1, task = thread + t NT.
@@ -398,7 +402,7 @@ __device__ __forceinline__ void syn_compute(const R *q, R *tl, R *th, R (&acc)[N
     for (int task = threadIdx.x; task < 2 * EXT * NR; task += NT) {
         const int half = task >= EXT * NR, s = task - half * EXT * NR, j = s % EXT, p0 = (s / EXT) * PS;
         const R *qa = q + (half * G::EXT + p0) * G::PQ + 9 - H + j, *qb = qa + 2 * G::EXT * G::PQ;
-        R e[PS], o[PS], eh[PS], oh[PS];   // low and high half apart: fewer roundings at the sum's size
+        R e[PS], o[PS], eh[PS], oh[PS];
 #pragma unroll
         for (int p = 0; p < PS; ++p) e[p] = o[p] = eh[p] = oh[p] = R(0);
 #pragma unroll
@@ -519,7 +523,7 @@ __global__ void __launch_bounds__(NT) k_sara_syn(const R *__restrict__ coef, con
 // in its shared memory, then sums an eighth of the tile's rows over the
 // cluster.  One CTA working through the 8 bases took 8 rounds of copy,
 // barrier and cold filter code (21 us at 512^2, 19 us at 256^2, 157 us at
-// 2048^2 with these tiles; the cluster takes 10, 6 and 100).  What bounds it
+// 2048^2 with these tiles; the cluster takes 10, 6 and 101).  What bounds it
 // now is the longest filter of a cluster and its two cluster barriers.
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
